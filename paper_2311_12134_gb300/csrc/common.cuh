@@ -260,6 +260,10 @@ int step_tc_chunk(const Unit* d_units, int n_units, int n_max, const char* fac_b
 int gemm_tc_chunk(const Unit* d_units, int n_units, int n_max, int k, char* fac_base, int32_t* stat,
                   cudaStream_t st);
 
+// Trailing update of the complex128 LU on the tensor cores, exact bf16 digit products (tc_gemm64.cu).
+int gemm64_tc_chunk(const Unit* d_units, int n_units, int n_max, int k, char* fac_base, int32_t* stat,
+                    cudaStream_t st);
+
 int existing_device_data(lsms_liz* liz, DeviceData** out);
 
 // Process-wide options (lsms_set_option).

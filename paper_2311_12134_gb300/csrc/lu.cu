@@ -10,9 +10,9 @@
 //                form U12 = L11^{-1} A12 (one warp per column); columns left
 //                of the panel are not swapped (L is kept as computed, LINPACK
 //                style),
-//   k_gemm       A22 -= L21 U12: register-tiled complex GEMM on the FP64 pipe
-//                (FP64 form); the complex64 form uses k_gemm_tc (tc_gemm.cu),
-//                the same update on the tensor cores.
+//   A22 -= L21 U12 on the tensor cores: k_gemm64_tc (tc_gemm64.cu, exact digit
+//                products) for complex128, k_gemm_tc (tc_gemm.cu, 3xTF32) for
+//                complex64.
 // Units of a chunk are sorted by n (largest first); each launch covers every
 // unit and units already finished return at once.  k_solve (FP64) and
 // k_solve_c64 (complex64) then run blocked forward/backward substitution; the
@@ -686,69 +686,6 @@ __global__ void __launch_bounds__(256) k_swap_trsm(const Unit* __restrict__ unit
   for (int i = 0; i < NB; ++i) Ac[k + i] = x[i];
 }
 
-// ------------------------------------------------------------------ trailing GEMM (SIMT)
-// Tile 64 x 64, K slices of 16; thread (ty, tx) owns rows ty + 16 r, columns tx + 16 c.
-template <typename R, int NB>
-__global__ void __launch_bounds__(256) k_gemm(const Unit* __restrict__ units, char* fac_base, int k,
-                                              int tiles_max) {
-  using C = Cx<R>;
-  const Unit u = units[blockIdx.y];
-  const int n = u.n;
-  const int t0 = k + NB;
-  const int mt = n - t0;
-  if (mt <= 0) return;
-  const int tiles = (mt + 63) >> 6;
-  const int ti = blockIdx.x / tiles_max, tj = blockIdx.x % tiles_max;
-  if (ti >= tiles || tj >= tiles) return;
-  C* A = reinterpret_cast<C*>(fac_base + u.fac_off);
-  const int row0 = t0 + 64 * ti, col0 = t0 + 64 * tj;
-  __shared__ C sA[16][64];
-  __shared__ C sB[16][65];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  C acc[4][4];
-#pragma unroll
-  for (int r = 0; r < 4; ++r)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) acc[r][c] = mk(R(0), R(0));
-  for (int ks = 0; ks < NB; ks += 16) {
-    for (int idx = threadIdx.x; idx < 16 * 64; idx += 256) {
-      const int i = idx & 63, kk = idx >> 6;
-      const int row = row0 + i;
-      sA[kk][i] = row < n ? A[(size_t)(k + ks + kk) * n + row] : mk(R(0), R(0));
-      const int kk2 = idx & 15, j = idx >> 4;
-      const int col = col0 + j;
-      sB[kk2][j] = col < n ? A[(size_t)col * n + k + ks + kk2] : mk(R(0), R(0));
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < 16; ++kk) {
-      C a[4], b[4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) a[r] = sA[kk][ty + 16 * r];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) b[c] = sB[kk][tx + 16 * c];
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) acc[r][c] = cfma(a[r], b[c], acc[r][c]);
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    const int col = col0 + tx + 16 * c;
-    if (col >= n) continue;
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int row = row0 + ty + 16 * r;
-      if (row < n) {
-        C* a = A + (size_t)col * n + row;
-        *a = csub(*a, acc[r][c]);
-      }
-    }
-  }
-}
-
 // ------------------------------------------------------------------ solve
 // X[i][c] -= sum_j A[i][k + j] sX[j][c] for rows i in [r0, r1): one thread per
 // (row, group of 4 right-hand sides); the NB column entries of A are loaded 8 at
@@ -1402,8 +1339,9 @@ int lu_factor_chunk(const Unit* d_units, int n_units, int n_max, char* fac_base,
       const int rc = gemm_tc_chunk(d_units, n_units, n_max, k, fac_base, stat, st);
       if (rc) return rc;
     } else {
-      const int tiles = (trail + 63) / 64;
-      LSMS_LAUNCH((k_gemm<R, NB>), dim3(tiles * tiles, n_units), dim3(256), 0, st, d_units, fac_base, k, tiles);
+      // complex128: exact digit products on the tensor cores (tc_gemm64.cu)
+      const int rc = gemm64_tc_chunk(d_units, n_units, n_max, k, fac_base, stat, st);
+      if (rc) return rc;
     }
   }
   // complex64: inverses of the diagonal blocks for the solves, L in the row order
