@@ -264,6 +264,10 @@ int gemm_tc_chunk(const Unit* d_units, int n_units, int n_max, int k, char* fac_
 int gemm64_tc_chunk(const Unit* d_units, int n_units, int n_max, int k, char* fac_base, int32_t* stat,
                     cudaStream_t st);
 
+// Solve L U X = P B in place on the X field (complex128, nrhs <= 32), row updates as the same digit products.
+int solve64_tc_chunk(const Unit* d_units, int n_units, const char* fac_base, char* ws, int nrhs, int32_t* stat,
+                     cudaStream_t st);
+
 int existing_device_data(lsms_liz* liz, DeviceData** out);
 
 // Process-wide options (lsms_set_option).

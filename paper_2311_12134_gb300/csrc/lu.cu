@@ -14,10 +14,9 @@
 //                products) for complex128, k_gemm_tc (tc_gemm.cu, 3xTF32) for
 //                complex64.
 // Units of a chunk are sorted by n (largest first); each launch covers every
-// unit and units already finished return at once.  k_solve (FP64) and
-// k_solve_c64 (complex64) then run blocked forward/backward substitution; the
-// forward sweep applies each panel's row swaps to the right-hand sides just
-// before that panel's block of L, so the right-hand sides come in unpermuted.
+// unit and units already finished return at once.  k_solve64_tc (FP64,
+// tc_gemm64.cu) and k_solve_c64 (complex64) then run blocked forward/backward
+// substitution.
 #include <algorithm>
 #include <type_traits>
 
@@ -28,70 +27,6 @@
 namespace lsms {
 
 template <typename R> struct LuCfg { static constexpr int NB = 32; };
-
-__device__ __forceinline__ double2 shfl2(double2 v, int src) {
-  return make_double2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
-}
-__device__ __forceinline__ float2 shfl2(float2 v, int src) {
-  return make_float2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
-}
-
-// The row interchanges of one factor panel (rows k + j <-> sp[j], j = 0..31 in
-// order; sp[j] = k + j for no interchange) applied to one column by one warp.
-// Lane j holds row k + j of the column in x on entry and exit; rows below the
-// panel that the interchanges reach are read and written in place.  When those
-// rows are all distinct (the usual case) each is read once up front and written
-// once at the end and the sequence runs in registers; repeated targets take the
-// sequential path through memory.
-template <typename C>
-__device__ __forceinline__ C panel_swaps(C x, C* col, const int* sp, int k, int lane) {
-  constexpr int NB = 32;
-  const int pj = sp[lane];
-  const bool outj = pj >= k + NB;
-  const unsigned same = __match_any_sync(0xffffffffu, outj ? pj : -1 - lane);
-  const bool fast = !__any_sync(0xffffffffu, outj && __popc(same) > 1);
-  if (fast) {
-    C y = outj ? col[pj] : x;
-#pragma unroll
-    for (int j = 0; j < NB; ++j) {
-      const int p = sp[j];
-      if (p == k + j) continue;
-      if (p < k + NB) {
-        const int b = p - k;
-        const C va = shfl2(x, j);
-        const C vb = shfl2(x, b);
-        if (lane == j) x = vb;
-        if (lane == b) x = va;
-      } else if (lane == j) {
-        const C t = y;
-        y = x;
-        x = t;
-      }
-    }
-    if (outj) col[pj] = y;
-  } else {
-#pragma unroll
-    for (int j = 0; j < NB; ++j) {
-      const int p = sp[j];
-      if (p == k + j) continue;
-      if (p < k + NB) {
-        const int b = p - k;
-        const C va = shfl2(x, j);
-        const C vb = shfl2(x, b);
-        if (lane == j) x = vb;
-        if (lane == b) x = va;
-      } else {
-        if (lane == j) {
-          const C t = col[p];
-          col[p] = x;
-          x = t;
-        }
-        __syncwarp();
-      }
-    }
-  }
-  return x;
-}
 
 // Asynchronous global -> shared copy of one complex element (cp.async: 8 bytes
 // for complex64, 16 for complex128); completed by cp.async.wait_all.
@@ -684,111 +619,6 @@ __global__ void __launch_bounds__(256) k_swap_trsm(const Unit* __restrict__ unit
   }
 #pragma unroll
   for (int i = 0; i < NB; ++i) Ac[k + i] = x[i];
-}
-
-// ------------------------------------------------------------------ solve
-// X[i][c] -= sum_j A[i][k + j] sX[j][c] for rows i in [r0, r1): one thread per
-// (row, group of 4 right-hand sides); the NB column entries of A are loaded 8 at
-// a time before use so that the loads overlap.
-template <typename R, int NB>
-__device__ __forceinline__ void update_rows(const Cx<R>* __restrict__ A, Cx<R>* X, const Cx<R> (*sX)[33], int n, int k,
-                                            int nbp, int r0, int r1, int nrhs, int tid, int nthr) {
-  using C = Cx<R>;
-  constexpr int G = 4;  // right-hand sides per thread
-  const int rows = r1 - r0;
-  if (rows <= 0) return;
-  const int ngrp = (nrhs + G - 1) / G;
-  for (int idx = tid; idx < rows * ngrp; idx += nthr) {
-    const int i = r0 + idx % rows, g = (idx / rows) * G;
-    C acc[G];
-#pragma unroll
-    for (int c = 0; c < G; ++c) acc[c] = (g + c < nrhs) ? X[(size_t)(g + c) * n + i] : mk(R(0), R(0));
-    for (int j0 = 0; j0 < nbp; j0 += 8) {
-      C l[8];
-#pragma unroll
-      for (int jj = 0; jj < 8; ++jj) l[jj] = (j0 + jj < nbp) ? A[(size_t)(k + j0 + jj) * n + i] : mk(R(0), R(0));
-#pragma unroll
-      for (int jj = 0; jj < 8; ++jj)
-#pragma unroll
-        for (int c = 0; c < G; ++c) acc[c] = cfms(l[jj], sX[j0 + jj][(g + c < nrhs) ? g + c : 0], acc[c]);
-    }
-#pragma unroll
-    for (int c = 0; c < G; ++c)
-      if (g + c < nrhs) X[(size_t)(g + c) * n + i] = acc[c];
-  }
-}
-
-// One CTA of 512 threads per unit: L y = P b (unit lower, each panel's swaps
-// applied just before its block), then U x = y, on the n x nrhs column-major
-// block X.  The NB x NB triangles are solved by warps taking columns in turn (lane = row, values
-// passed by shuffles); the rows below/above are updated by the whole CTA.
-template <typename R, int NB>
-__global__ void __launch_bounds__(512, 2) k_solve(const Unit* __restrict__ units, const char* fac_base, char* ws,
-                                                int which, int nrhs, const int32_t* done) {
-  using C = Cx<R>;
-  static_assert(NB == 32, "one lane per row of the diagonal block");
-  const Unit u = units[blockIdx.x];
-  if (done && done[u.stat_off]) return;
-  const int n = u.n;
-  if (n == 0) return;  // an unused FP64 fallback slot
-  const C* A = reinterpret_cast<const C*>(fac_base + u.fac_off);
-  C* X = reinterpret_cast<C*>(ws + (which == RHS_X ? u.x_off : u.x32_off));
-  const int32_t* piv = reinterpret_cast<const int32_t*>(fac_base + u.piv_off);
-  __shared__ C sT[NB][NB + 1];
-  __shared__ C sX[NB][33];
-  __shared__ int sp[NB];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int nthr = blockDim.x;
-  // forward
-  for (int k = 0; k < n; k += NB) {
-    const int nbp = min(NB, n - k);
-    for (int idx = tid; idx < NB * NB; idx += nthr) {
-      const int i = idx % NB, j = idx / NB;
-      sT[i][j] = (i < nbp && j < nbp) ? A[(size_t)(k + j) * n + k + i] : mk(R(0), R(0));
-    }
-    if (tid < NB) sp[tid] = tid < nbp ? piv[k + tid] : k + tid;
-    __syncthreads();
-    for (int col = warp; col < nrhs; col += nthr >> 5) {
-      C x = lane < nbp ? X[(size_t)col * n + k + lane] : mk(R(0), R(0));
-      x = panel_swaps(x, X + (size_t)col * n, sp, k, lane);
-      for (int j = 0; j < nbp - 1; ++j) {
-        const C xj = shfl2(x, j);
-        if (lane > j) x = cfms(sT[lane][j], xj, x);
-      }
-      if (lane < nbp) {
-        X[(size_t)col * n + k + lane] = x;
-        sX[lane][col] = x;
-      }
-    }
-    __syncthreads();
-    update_rows<R, NB>(A, X, sX, n, k, nbp, k + nbp, n, nrhs, tid, nthr);
-    __syncthreads();
-  }
-  // backward
-  const int last = ((n - 1) / NB) * NB;
-  for (int k = last; k >= 0; k -= NB) {
-    const int nbp = min(NB, n - k);
-    for (int idx = tid; idx < NB * NB; idx += nthr) {
-      const int i = idx % NB, j = idx / NB;
-      sT[i][j] = (i < nbp && j < nbp) ? A[(size_t)(k + j) * n + k + i] : mk(R(1), R(0));
-    }
-    __syncthreads();
-    for (int col = warp; col < nrhs; col += nthr >> 5) {
-      C x = lane < nbp ? X[(size_t)col * n + k + lane] : mk(R(0), R(0));
-      for (int j = nbp - 1; j >= 0; --j) {
-        if (lane == j) x = cmul(x, crcp(sT[j][j]));
-        const C xj = shfl2(x, j);
-        if (lane < j) x = cfms(sT[lane][j], xj, x);
-      }
-      if (lane < nbp) {
-        X[(size_t)col * n + k + lane] = x;
-        sX[lane][col] = x;
-      }
-    }
-    __syncthreads();
-    update_rows<R, NB>(A, X, sX, n, k, nbp, 0, k, nrhs, tid, nthr);
-    __syncthreads();
-  }
 }
 
 // ------------------------------------------------------------------ complex64 solve
@@ -1468,7 +1298,7 @@ int lu_solve_chunk(const Unit* d_units, int n_units, int n_max, const char* fac_
 #undef LSMS_SOLVE
     }
   } else {
-    LSMS_LAUNCH((k_solve<R, NB>), dim3(n_units), dim3(512), 0, st, d_units, fac_base, ws, which_rhs, nrhs, done);
+    return solve64_tc_chunk(d_units, n_units, fac_base, ws, nrhs, stat, st);
   }
   return LSMS_OK;
 }

@@ -36,20 +36,21 @@ namespace lsms {
 
 namespace oz {
 
-constexpr int ND = 7;                 // digits per operand, classes per accumulator
 constexpr int NB = 32;                // complex panel width
 constexpr int TM = 128;               // rows per CTA (TMEM lanes)
 constexpr int NCC = 16;               // complex columns per tile
 constexpr int NR = 2 * NCC;           // real accumulator columns per class: [Re | Im]
 constexpr int NT = 512;               // threads: (row, 8-column chunk) of L21; (column, row) of a U12 tile
+constexpr int kGemmDigits = 7;        // digits per operand, classes per accumulator
+constexpr int kSolveDigits = 8;       // (the right-hand sides spread over more orders of magnitude, see there)
 constexpr int PLANE_A = TM * 128;     // one digit of A: 64 real K x 2 bytes per row, 128-byte swizzle
 constexpr int PLANE_B = NR * 128;
-constexpr int STAGE_B = ND * PLANE_B;
-constexpr int SMEM_BYTES = ND * PLANE_A + 2 * STAGE_B + 4 * TM * 4 + 4 * NCC * 4 + 64 + 1024;
-constexpr uint32_t ACC_COLS = 256;    // columns between the two accumulators (ND * NR = 224 used)
+template <int ND>
+constexpr int kGemmSmem = ND * PLANE_A + 2 * ND * PLANE_B + 4 * TM * 4 + 4 * NCC * 4 + 64 + 1024;
+constexpr uint32_t ACC_COLS = 256;    // columns between the two accumulators (ND * NR used)
 constexpr uint32_t TMEM_COLS = 512;
 constexpr long long kWaitLimit = 1ll << 24;  // bounded mbarrier wait (polls)
-static_assert(ND * NR <= (int)ACC_COLS && NT == TM * 4 && NT == NCC * NB, "tile shape");
+static_assert(NT == TM * 4 && NT == NCC * NB, "tile shape");
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -98,59 +99,94 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, float* v) {  // complet
                : "r"(taddr));
 }
 
+__device__ __forceinline__ void tmem_ld2(uint32_t taddr, float* v) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];" : "=f"(v[0]), "=f"(v[1]) : "r"(taddr));
+}
+
+// |digit 0| <= 2^top_bits: seven digits of a value scaled to 2^7 (55 fraction and integer bits
+// in 7 bytes), or eight of a value scaled to 2^6 (62 bits in 8 bytes).
+template <int ND>
+__host__ __device__ constexpr int top_bits() {
+  static_assert(ND == 7 || ND == 8, "digits per operand");
+  return ND == 7 ? 7 : 6;
+}
+
+// One thread: the digit products (per 16 K, one instruction per digit of A) of a 128 x 16
+// complex tile with 32 complex K, committed to an mbarrier.
+template <int ND>
+__device__ __forceinline__ void issue_tile(uint32_t d, uint32_t a0, uint32_t b0, uint32_t mbar) {
+#pragma unroll
+  for (int ks = 0; ks < 4; ++ks)
+#pragma unroll
+    for (int s = 0; s < ND; ++s)
+      mma_bf16(d + (uint32_t)(s * NR), make_desc(a0 + s * PLANE_A + ks * 32), make_desc(b0 + ks * 32),
+               make_idesc(TM, NR * (ND - s)), (ks | s) ? 1u : 0u);
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar) : "memory");
+}
+
+// Scale of class_sum's integers for the exponent fields eL, eU of the row and column maxima:
+// class 0 weighs 2^(eL + eU - 2 * 1022 - 2 top_bits), the integers count 2^-40 of it.  NaN when
+// one of the two stands for a non-finite value.
+template <int ND>
+__device__ __forceinline__ double product_scale(int el, int eu) {
+  const int ex = el + eu - 2 * 1022 - 2 * top_bits<ND>() - 40 + 1023;
+  return __hiloint2double(ex <= 0 ? 0 : (ex >= 0x7ff ? 0x7ff80000 : ex << 20), 0);
+}
+
 __device__ __forceinline__ int exp_field(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
 
-// rint(v 2^(55 - E)) plus 128 in each of the six low bytes, E = emax - 1022 (|v| < 2^E when
-// v's exponent field is at most emax): bytes 0..5 are digits 6..1 plus 128, the bits from 48
-// up digit 0.  Subnormals count as zero (below 2^-1022).
+// rint(v 2^(8 (ND - 1) + top_bits - E)) plus 128 in each of its ND - 1 low bytes, E = emax - 1022
+// (|v| < 2^E when v's exponent field is at most emax): the low bytes are digits ND - 1 .. 1 plus
+// 128, what is above them digit 0.  Subnormals count as zero (below 2^-1022).
+template <int ND>
 __device__ __forceinline__ long long biased_digits(double v, int emax) {
   const long long b = __double_as_longlong(v);
   const int e = (int)(b >> 52) & 0x7ff;
   const long long m = e ? ((b & 0xfffffffffffffll) | 0x10000000000000ll) : 0ll;
-  const int sh = e - emax + 2;  // <= 2
+  const int sh = e - emax + (ND == 7 ? 2 : 9);  // m 2^(e - 1075) 2^(..): at most 2 or 9 to the left
   const int r = min(max(-sh, 0), 62);
   const long long half = r ? 1ll << (r - 1) : 0ll;
   const long long mag = ((m << max(sh, 0)) + half) >> r;
-  return (b < 0 ? -mag : mag) + 0x0000808080808080ll;
+  return (b < 0 ? -mag : mag) + (ND == 7 ? 0x0000808080808080ll : 0x0080808080808080ll);
 }
 
 // Digit s of a biased value as the bits of a float (an integer of at most 8 significant
 // bits: its upper 16 bits are the bf16 value, exactly).
-template <int s>
+template <int ND, int s>
 __device__ __forceinline__ uint32_t digit_bits(long long j) {
-  if constexpr (s == 0) {
-    const uint32_t hi = (uint32_t)((unsigned long long)j >> 32) ^ 0x80000000u;
-    return __float_as_uint(__uint_as_float(__byte_perm(hi, 0x4B000000u, 0x7432)) - 8421376.f);
+  const uint32_t hi = (uint32_t)((unsigned long long)j >> 32);
+  if constexpr (s == 0 && ND == 7) {  // the 16 bits above the bytes
+    return __float_as_uint(__uint_as_float(__byte_perm(hi ^ 0x80000000u, 0x4B000000u, 0x7432)) - 8421376.f);
   } else {
-    const uint32_t w = s <= 2 ? (uint32_t)((unsigned long long)j >> 32) : (uint32_t)j;
-    constexpr int byte = s <= 2 ? 2 - s : 6 - s;
-    return __float_as_uint(__uint_as_float(__byte_perm(w, 0x4B000000u, 0x7440 + byte)) - 8388736.f);
+    constexpr int byte = ND - 1 - s;
+    const uint32_t w = byte >= 4 ? (s == 0 ? hi ^ 0x80000000u : hi) : (uint32_t)j;
+    return __float_as_uint(__uint_as_float(__byte_perm(w, 0x4B000000u, 0x7440 + (byte & 3))) - 8388736.f);
   }
 }
 
 // One digit plane of A: the 8 columns of this thread's chunk, real parts to 16-byte unit
 // `chunk` of its row, imaginary parts to unit 4 + chunk.
-template <int s>
+template <int ND, int s>
 __device__ __forceinline__ void put_a(uint8_t* sA, int row, int chunk, const long long (&jr)[8], const long long (&ji)[8]) {
   uint4 re, im;
   uint32_t* pr = &re.x;
   uint32_t* pi = &im.x;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    pr[q] = __byte_perm(digit_bits<s>(jr[2 * q]), digit_bits<s>(jr[2 * q + 1]), 0x7632);
-    pi[q] = __byte_perm(digit_bits<s>(ji[2 * q]), digit_bits<s>(ji[2 * q + 1]), 0x7632);
+    pr[q] = __byte_perm(digit_bits<ND, s>(jr[2 * q]), digit_bits<ND, s>(jr[2 * q + 1]), 0x7632);
+    pi[q] = __byte_perm(digit_bits<ND, s>(ji[2 * q]), digit_bits<ND, s>(ji[2 * q + 1]), 0x7632);
   }
   uint8_t* p = sA + s * PLANE_A + row * 128;
   *reinterpret_cast<uint4*>(p + ((chunk ^ (row & 7)) << 4)) = re;
   *reinterpret_cast<uint4*>(p + (((4 + chunk) ^ (row & 7)) << 4)) = im;
-  if constexpr (s + 1 < ND) put_a<s + 1>(sA, row, chunk, jr, ji);
+  if constexpr (s + 1 < ND) put_a<ND, s + 1>(sA, row, chunk, jr, ji);
 }
 
 // One digit plane of B, U12(k, c): row c (real output) holds Re at K k and -Im at K 32 + k,
 // row 16 + c (imaginary output) Im and Re.
-template <int t>
+template <int ND, int t>
 __device__ __forceinline__ void put_b(uint8_t* sB, int c, int k, long long jr, long long ji) {
-  const uint32_t re = digit_bits<t>(jr) >> 16, im = digit_bits<t>(ji) >> 16;
+  const uint32_t re = digit_bits<ND, t>(jr) >> 16, im = digit_bits<ND, t>(ji) >> 16;
   const int u = k >> 3, off = (k & 7) * 2, x = c & 7;
   uint8_t* p = sB + t * PLANE_B + c * 128;
   uint8_t* q = p + NCC * 128;  // (16 + c) & 7 == c & 7
@@ -158,30 +194,36 @@ __device__ __forceinline__ void put_b(uint8_t* sB, int c, int k, long long jr, l
   *reinterpret_cast<unsigned short*>(p + (((4 + u) ^ x) << 4) + off) = (unsigned short)(im ^ 0x8000u);
   *reinterpret_cast<unsigned short*>(q + ((u ^ x) << 4) + off) = (unsigned short)im;
   *reinterpret_cast<unsigned short*>(q + (((4 + u) ^ x) << 4) + off) = (unsigned short)re;
-  if constexpr (t + 1 < ND) put_b<t + 1>(sB, c, k, jr, ji);
+  if constexpr (t + 1 < ND) put_b<ND, t + 1>(sB, c, k, jr, ji);
 }
 
-// The class sums of one real value as a fixed-point integer in units of 2^-40 of the class-0
-// weight: exact but for the last class, rounded to that unit (2^-54 of the two scales).
-__device__ __forceinline__ long long class_sum(const float (&v)[ND]) {
+// The class sums of one real value as a number in units of 2^-40 of the class-0 weight, rounded
+// to FP64: classes 0..5 exactly in 64-bit integers; of seven digits the last class rounded to
+// that unit (2^-54 of the two scales), of eight the last two added in FP64.
+template <int ND>
+__device__ __forceinline__ double class_sum(const float (&v)[ND]) {
   int i[ND];
 #pragma unroll
   for (int g = 0; g < ND; ++g) i[g] = __float2int_rn(v[g]);
-  const int a = i[0] * 256 + i[1];                          // below 2^29
-  const int b = i[2] * 256 + i[3];                          // below 2^30
-  const int c = i[4] * 256 + i[5] + ((i[6] + 128) >> 8);    // below 2^31
-  return ((long long)a << 32) + (long long)b * 65536 + c;
+  const int a = i[0] * 256 + i[1];  // below 2^29
+  const int b = i[2] * 256 + i[3];  // below 2^30
+  int c = i[4] * 256 + i[5];        // below 2^31
+  if constexpr (ND == 7) c += (i[6] + 128) >> 8;
+  const double s = (double)(((long long)a << 32) + (long long)b * 65536 + c);
+  if constexpr (ND == 7) return s;
+  else return fma((double)(i[6] * 256 + i[7]), 0x1p-16, s);
 }
 
 }  // namespace oz
 
 // grid (row tiles of 128, n_units, column splits), block 512, dynamic smem
-// oz::SMEM_BYTES (one CTA per SM).  One CTA per 128-row block of a unit's trailing
+// oz::kGemmSmem (one CTA per SM).  One CTA per 128-row block of a unit's trailing
 // matrix walks its share of the 16-column tiles: L21's digit planes are staged
 // once; the digits of the next tile's U12 are staged and its product issued (into
 // the other accumulator) before the epilogue of the current tile, which the
 // tensor cores therefore overlap.  Waits on the tensor core are bounded
 // (LSMS_UNIT_TIMEOUT).  A row or column with a non-finite value gives NaN.
+template <int ND>
 __global__ void __launch_bounds__(oz::NT, 1) k_gemm64_tc(const Unit* __restrict__ units, char* fac_base, int k,
                                                          int32_t* stat) {
   using namespace oz;
@@ -197,6 +239,8 @@ __global__ void __launch_bounds__(oz::NT, 1) k_gemm64_tc(const Unit* __restrict_
   const int j0 = blockIdx.z * per, j1 = min(tiles, j0 + per);
   if (j0 >= j1) return;
   double2* A = reinterpret_cast<double2*>(fac_base + u.fac_off);
+  constexpr int STAGE_B = ND * PLANE_B;
+  static_assert(ND * NR <= (int)ACC_COLS, "classes of an accumulator");
 
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -229,7 +273,7 @@ __global__ void __launch_bounds__(oz::NT, 1) k_gemm64_tc(const Unit* __restrict_
     e = __reduce_max_sync(0xffffffffu, e);
     // (slots of 4: a slower warp may still read the exponents of tile j - 2)
     if (lane == 0) sCexp[(j & 3) * NCC + warp] = e == 0x7ff ? 1 << 14 : e;
-    put_b<0>(sB + (j & 1) * STAGE_B, warp, lane, biased_digits(v.x, e), biased_digits(v.y, e));
+    put_b<ND, 0>(sB + (j & 1) * STAGE_B, warp, lane, biased_digits<ND>(v.x, e), biased_digits<ND>(v.y, e));
   };
   double2 uv = load_u(j0);
 
@@ -250,10 +294,10 @@ __global__ void __launch_bounds__(oz::NT, 1) k_gemm64_tc(const Unit* __restrict_
     long long jr[8], ji[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      jr[q] = biased_digits(v[q].x, e);
-      ji[q] = biased_digits(v[q].y, e);
+      jr[q] = biased_digits<ND>(v[q].x, e);
+      ji[q] = biased_digits<ND>(v[q].y, e);
     }
-    put_a<0>(sA, ar, chunk, jr, ji);
+    put_a<ND, 0>(sA, ar, chunk, jr, ji);
   }
 
   // epilogue: TMEM lane (warp % 4) * 32 + lane = row, complex columns 4 (warp / 4) .. + 3
@@ -262,19 +306,6 @@ __global__ void __launch_bounds__(oz::NT, 1) k_gemm64_tc(const Unit* __restrict_
   int rexp = max(max(sRexp[er], sRexp[TM + er]), max(sRexp[2 * TM + er], sRexp[3 * TM + er]));
   if (rexp == 0x7ff) rexp = 1 << 14;
 
-  auto issue = [&](int j, uint32_t tmem) {  // one thread: the 28 products of a tile
-    const uint32_t d = tmem + (uint32_t)(j & 1) * ACC_COLS;
-    const uint32_t a0 = smem_u32(sA), b0 = smem_u32(sB + (j & 1) * STAGE_B);
-#pragma unroll
-    for (int ks = 0; ks < 4; ++ks)
-#pragma unroll
-      for (int s = 0; s < ND; ++s)
-        mma_bf16(d + (uint32_t)(s * NR), make_desc(a0 + s * PLANE_A + ks * 32), make_desc(b0 + ks * 32),
-                 make_idesc(TM, NR * (ND - s)), (ks | s) ? 1u : 0u);
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                     smem_u32(mbar + (j & 1)))
-                 : "memory");
-  };
   // stage U12 of tile j (its buffer and accumulator free: tile j - 2 is done) and issue its product
   uint32_t tmem = 0;
   auto launch_tile = [&](int j) {
@@ -284,7 +315,10 @@ __global__ void __launch_bounds__(oz::NT, 1) k_gemm64_tc(const Unit* __restrict_
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     tmem = *tslot;
-    if (tid == 0) issue(j - j0, tmem);
+    if (tid == 0) {
+      const int b = (j - j0) & 1;
+      issue_tile<ND>(tmem + (uint32_t)b * ACC_COLS, smem_u32(sA), smem_u32(sB + b * STAGE_B), smem_u32(mbar + b));
+    }
     if (j + 1 < j1) uv = load_u(j + 1);
   };
 
@@ -330,10 +364,8 @@ __global__ void __launch_bounds__(oz::NT, 1) k_gemm64_tc(const Unit* __restrict_
         vr[g] = re[g][c];
         vi[g] = im[g][c];
       }
-      // L U = class sum x 2^(eL - 1022 + eU - 1022 - 14 - 40)
-      const int ex = rexp + sCexp[(it & 3) * NCC + ec + c] - 1075;
-      const double sc = __hiloint2double(ex <= 0 ? 0 : (ex >= 0x7ff ? 0x7ff80000 : ex << 20), 0);
-      const double2 r = make_double2(fma(-(double)class_sum(vr), sc, cv[c].x), fma(-(double)class_sum(vi), sc, cv[c].y));
+      const double sc = product_scale<ND>(rexp, sCexp[(it & 3) * NCC + ec + c]);
+      const double2 r = make_double2(fma(-class_sum<ND>(vr), sc, cv[c].x), fma(-class_sum<ND>(vi), sc, cv[c].y));
       if (crow < n && c0 + c < n) A[(size_t)(c0 + c) * n + crow] = r;
     }
   }
@@ -356,7 +388,8 @@ int gemm64_tc_chunk(const Unit* d_units, int n_units, int n_max, int k, char* fa
                     cudaStream_t st) {
   static bool attr_set = false;
   if (!attr_set) {
-    LSMS_CUDA_TRY(cudaFuncSetAttribute(k_gemm64_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, oz::SMEM_BYTES));
+    LSMS_CUDA_TRY(cudaFuncSetAttribute(k_gemm64_tc<oz::kGemmDigits>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       oz::kGemmSmem<oz::kGemmDigits>));
     attr_set = true;
   }
   const int mt = n_max - k - oz::NB;
@@ -366,7 +399,346 @@ int gemm64_tc_chunk(const Unit* d_units, int n_units, int n_max, int k, char* fa
   // L21 costs about as much as two tiles)
   const int want = 2 * 152 / std::max(1, rows * n_units);
   const int split = std::max(1, std::min(want, tiles / 4));
-  LSMS_LAUNCH(k_gemm64_tc, dim3(rows, n_units, split), dim3(oz::NT), oz::SMEM_BYTES, st, d_units, fac_base, k, stat);
+  LSMS_LAUNCH(k_gemm64_tc<oz::kGemmDigits>, dim3(rows, n_units, split), dim3(oz::NT),
+              oz::kGemmSmem<oz::kGemmDigits>, st, d_units, fac_base, k, stat);
+  return LSMS_OK;
+}
+
+}  // namespace lsms
+
+// ------------------------------------------------------------------ solve
+namespace lsms {
+
+__device__ __forceinline__ double2 shfl2(double2 v, int src) {
+  return make_double2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
+}
+
+// The row interchanges of one factor panel (rows k + j <-> sp[j], j = 0..31 in
+// order; sp[j] = k + j for no interchange) applied to one column by one warp.
+// Lane j holds row k + j of the column in x on entry and exit; rows below the
+// panel that the interchanges reach are read and written in place.  When those
+// rows are all distinct (the usual case) each is read once up front and written
+// once at the end and the sequence runs in registers; repeated targets take the
+// sequential path through memory.
+template <typename C>
+__device__ __forceinline__ C panel_swaps(C x, C* col, const int* sp, int k, int lane) {
+  constexpr int NB = 32;
+  const int pj = sp[lane];
+  const bool outj = pj >= k + NB;
+  const unsigned same = __match_any_sync(0xffffffffu, outj ? pj : -1 - lane);
+  const bool fast = !__any_sync(0xffffffffu, outj && __popc(same) > 1);
+  if (fast) {
+    C y = outj ? col[pj] : x;
+#pragma unroll
+    for (int j = 0; j < NB; ++j) {
+      const int p = sp[j];
+      if (p == k + j) continue;
+      if (p < k + NB) {
+        const int b = p - k;
+        const C va = shfl2(x, j);
+        const C vb = shfl2(x, b);
+        if (lane == j) x = vb;
+        if (lane == b) x = va;
+      } else if (lane == j) {
+        const C t = y;
+        y = x;
+        x = t;
+      }
+    }
+    if (outj) col[pj] = y;
+  } else {
+#pragma unroll
+    for (int j = 0; j < NB; ++j) {
+      const int p = sp[j];
+      if (p == k + j) continue;
+      if (p < k + NB) {
+        const int b = p - k;
+        const C va = shfl2(x, j);
+        const C vb = shfl2(x, b);
+        if (lane == j) x = vb;
+        if (lane == b) x = va;
+      } else {
+        if (lane == j) {
+          const C t = col[p];
+          col[p] = x;
+          x = t;
+        }
+        __syncwarp();
+      }
+    }
+  }
+  return x;
+}
+
+namespace oz {
+
+template <int ND>
+constexpr int kSolveSmem = ND * (PLANE_A + PLANE_B) + 3 * 4 * TM * 4 + NCC * 4 + 32 + NB * (NB + 1) * 16 +
+                           NB * (NCC + 1) * 16 + NB * 16 + 1024;
+
+}  // namespace oz
+
+// L y = P b (unit lower; each panel's row swaps applied just before its block), then
+// U x = y, in place on 16 columns (slice blockIdx.y) of the unit's n x nrhs
+// complex128 block X.  grid (n_units, ceil(nrhs / 16)), block 512, dynamic smem
+// oz::kSolveSmem (one CTA per SM).  Per 32-row block:
+//   the 32 x 32 triangle in FP64, 8 rows at a time: four warps substitute within
+//   8 x 8 (4 columns x 8 rows a warp), then all threads update the block's other
+//   rows; the diagonal's reciprocals are formed once per block by one warp;
+//   the rows below (above, going back) take X -= L y (U x) as digit products, 128
+//   rows at a time: A = the factor's rows (loaded a tile ahead, split when the
+//   previous tile's products are done), B = the solved block, split once; the
+//   epilogue of a tile runs under the products of the next.
+// Eight digits here: the rows of one solved block spread over orders of magnitude
+// (small high-l components meet large t^-1 entries), and with seven the tau error
+// rose by up to a third; with eight it is no larger than that of FP64 row updates
+// (6.1e-14 against 6.1e-14 at n = 2192, 1.43e-13 against 1.43e-13 at n = 688).
+// What bounds it: splitting the factor (each value serves 16 columns only, about
+// 0.7 clocks of integer work per SM and value) and the FP64 triangle.  Measured:
+// 216 matrices of n = 688, 16 columns: 4.15 ms against 19.8 ms with the row updates
+// on the FP64 pipe and a division per diagonal element and column; 20 matrices of
+// n = 160 0.24 against 1.00 ms.
+template <int ND>
+__global__ void __launch_bounds__(oz::NT, 1) k_solve64_tc(const Unit* __restrict__ units, const char* fac_base,
+                                                          char* ws, int nrhs, int32_t* stat) {
+  using namespace oz;
+  const Unit u = units[blockIdx.x];
+  const int n = u.n;
+  if (n == 0) return;  // an unused FP64 fallback slot
+  const double2* A = reinterpret_cast<const double2*>(fac_base + u.fac_off);
+  const int32_t* piv = reinterpret_cast<const int32_t*>(fac_base + u.piv_off);
+  const int cofs = blockIdx.y * NCC, ncol = min(NCC, nrhs - cofs);
+  double2* X = reinterpret_cast<double2*>(ws + u.x_off) + (size_t)cofs * n;
+  constexpr int STAGE_B = ND * PLANE_B;
+
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  uint8_t* sA = smem;
+  uint8_t* sB = sA + ND * PLANE_A;
+  double2(*sT)[NB + 1] = reinterpret_cast<double2(*)[NB + 1]>(sB + STAGE_B);      // the diagonal block
+  double2(*sX)[NCC + 1] = reinterpret_cast<double2(*)[NCC + 1]>(sT + NB);         // its rows of X
+  double2* sD = reinterpret_cast<double2*>(sX + NB);                              // reciprocals of U's diagonal
+  int* sRexp = reinterpret_cast<int*>(sD + NB);                                   // [3][4][TM], slot = tile % 3
+  int* sCexp = sRexp + 3 * 4 * TM;                                                // [NCC]
+  uint64_t* mbar = reinterpret_cast<uint64_t*>(sCexp + NCC);
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 1);
+  __shared__ int sp[NB];
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
+                 "r"(TMEM_COLS));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  if (tid == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(mbar)));
+    asm volatile("fence.mbarrier_init.release.cluster;");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *tslot;
+
+  const int ar = tid & (TM - 1), chunk = tid >> 7;                 // A: row, chunk of 8 columns
+  const int er = (warp & 3) * 32 + lane, ec = (warp >> 2) * 4;     // epilogue: TMEM lane, first column
+  int issued = 0;  // products committed so far; each is waited for before the next is issued
+  bool ok = true;
+
+  // products `issued - 1` complete (bounded); CTA-uniform, also the barrier of what came before
+  auto wait_products = [&]() -> bool {
+    bool w = true;
+    if (warp == 0 && issued > 0) {
+      w = false;
+      for (long long q = 0; q < kWaitLimit; ++q)
+        if (mbar_try_wait(smem_u32(mbar), (uint32_t)((issued - 1) & 1))) {
+          w = true;
+          break;
+        }
+    }
+    w = __syncthreads_and(w);
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    return w;
+  };
+  // X[row0 + er, ec ..] -= the products of the block's tile t
+  auto epilogue = [&](int row0, int r1, int t, const double2 (&cv)[4]) {
+    const int row = row0 + er;
+    const int* re4 = sRexp + (t % 3) * 4 * TM + er;
+    int rexp = max(max(re4[0], re4[TM]), max(re4[2 * TM], re4[3 * TM]));
+    if (rexp == 0x7ff) rexp = 1 << 14;
+    const uint32_t base = tmem + (uint32_t)(t & 1) * ACC_COLS + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)ec;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      float re[ND][2], im[ND][2];
+#pragma unroll
+      for (int g = 0; g < ND; ++g) {
+        tmem_ld2(base + (uint32_t)(g * NR + 2 * h), re[g]);
+        tmem_ld2(base + (uint32_t)(g * NR + NCC + 2 * h), im[g]);
+      }
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        float vr[ND], vi[ND];
+#pragma unroll
+        for (int g = 0; g < ND; ++g) {
+          vr[g] = re[g][c];
+          vi[g] = im[g][c];
+        }
+        const int col = ec + 2 * h + c;
+        const double sc = product_scale<ND>(rexp, sCexp[col]);
+        const double2 x = cv[2 * h + c];
+        if (row < r1 && col < ncol)
+          X[(size_t)col * n + row] =
+              make_double2(fma(-class_sum<ND>(vr), sc, x.x), fma(-class_sum<ND>(vi), sc, x.y));
+      }
+    }
+  };
+
+  const int nb = (n + NB - 1) / NB;
+  for (int step = 0; step < 2 * nb && ok; ++step) {
+    const bool fwd = step < nb;
+    const int k = NB * (fwd ? step : 2 * nb - 1 - step);
+    const int nbp = min(NB, n - k);
+    const int r0 = fwd ? k + nbp : 0, r1 = fwd ? n : k;  // rows to update
+    // the first tile's factor rows are requested before the triangle is solved
+    double2 v[8];
+    auto load_a = [&](int row0) {
+      const int row = row0 + ar;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int c = chunk * 8 + q;
+        v[q] = (row < r1 && c < nbp) ? A[(size_t)(k + c) * n + row] : make_double2(0.0, 0.0);
+      }
+    };
+    if (r0 < r1) load_a(r0);
+    for (int idx = tid; idx < NB * NB; idx += NT) {
+      const int i = idx % NB, j = idx / NB;
+      sT[i][j] = (i < nbp && j < nbp) ? A[(size_t)(k + j) * n + k + i] : make_double2(i == j ? 1.0 : 0.0, 0.0);
+    }
+    if (tid < NB) {
+      if (fwd) sp[tid] = tid < nbp ? piv[k + tid] : k + tid;
+      else sD[tid] = crcp(tid < nbp ? A[(size_t)(k + tid) * n + k + tid] : make_double2(1.0, 0.0));
+    }
+    __syncthreads();
+    {
+      const bool live = warp < ncol;
+      double2 x = make_double2(0.0, 0.0);
+      if (live) {
+        if (lane < nbp) x = X[(size_t)warp * n + k + lane];
+        if (fwd) x = panel_swaps(x, X + (size_t)warp * n, sp, k, lane);
+      }
+      sX[lane][warp] = x;
+    }
+    __syncthreads();
+    for (int bb = 0; bb < 4; ++bb) {
+      const int b0 = 8 * (fwd ? bb : 3 - bb);
+      if (warp < 4) {
+        const int c = 4 * warp + (lane >> 3), r = lane & 7, i = b0 + r;
+        double2 x = sX[i][c];
+        if (fwd) {
+#pragma unroll
+          for (int j = 0; j < 7; ++j) {
+            const double2 xj = shfl2(x, (lane & 24) + j);
+            if (r > j) x = cfms(sT[i][b0 + j], xj, x);
+          }
+        } else {
+#pragma unroll
+          for (int j = 7; j >= 0; --j) {
+            if (r == j) x = cmul(x, sD[i]);
+            const double2 xj = shfl2(x, (lane & 24) + j);
+            if (r < j) x = cfms(sT[i][b0 + j], xj, x);
+          }
+        }
+        sX[i][c] = x;
+      }
+      __syncthreads();
+      if (bb < 3) {
+        const int c = tid & 15, q = tid >> 4;
+        const int i = fwd ? b0 + 8 + q : q;
+        if (i < (fwd ? NB : b0)) {
+          double2 x = sX[i][c];
+#pragma unroll
+          for (int jj = 0; jj < 8; ++jj) {
+            const int j = b0 + (fwd ? jj : 7 - jj);
+            x = cfms(sT[i][j], sX[j][c], x);
+          }
+          sX[i][c] = x;
+        }
+        __syncthreads();
+      }
+    }
+    {
+      // the solved block: to X, and its digits into B (warp = column, lane = row; columns beyond
+      // ncol are zero)
+      const double2 y = sX[lane][warp];
+      if (warp < ncol && lane < nbp) X[(size_t)warp * n + k + lane] = y;
+      if (r0 < r1) {
+        const int e = __reduce_max_sync(0xffffffffu, max(exp_field(y.x), exp_field(y.y)));
+        if (lane == 0) sCexp[warp] = e == 0x7ff ? 1 << 14 : e;
+        put_b<ND, 0>(sB, warp, lane, biased_digits<ND>(y.x, e), biased_digits<ND>(y.y, e));
+      }
+    }
+    int t = 0;
+    double2 cv[4];
+    for (int row0 = r0; row0 < r1 && ok; row0 += TM, ++t) {
+      int e = 0;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) e = max(e, max(exp_field(v[q].x), exp_field(v[q].y)));
+      int* rexp = sRexp + (t % 3) * 4 * TM;  // a slower warp may still read tile t - 2's
+      rexp[chunk * TM + ar] = e;
+      if (!(ok = wait_products())) break;  // A free, the exponents visible
+      e = max(max(rexp[ar], rexp[TM + ar]), max(rexp[2 * TM + ar], rexp[3 * TM + ar]));
+      {
+        long long jr[8], ji[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          jr[q] = biased_digits<ND>(v[q].x, e);
+          ji[q] = biased_digits<ND>(v[q].y, e);
+        }
+        put_a<ND, 0>(sA, ar, chunk, jr, ji);
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncthreads();
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      if (tid == 0) {
+        issue_tile<ND>(tmem + (uint32_t)(t & 1) * ACC_COLS, smem_u32(sA), smem_u32(sB), smem_u32(mbar));
+      }
+      ++issued;
+      if (row0 + TM < r1) load_a(row0 + TM);
+      if (t > 0) epilogue(row0 - TM, r1, t - 1, cv);
+      const int row = row0 + er;
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        cv[c] = (row < r1 && ec + c < ncol) ? X[(size_t)(ec + c) * n + row] : make_double2(0.0, 0.0);
+    }
+    if (t > 0 && ok && (ok = wait_products())) epilogue(r0 + (t - 1) * TM, r1, t - 1, cv);
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();  // X current for the next block, B and the accumulators free
+  }
+  if (!ok && tid == 0) {
+    atomicOr(&stat[u.stat_off], LSMS_UNIT_TIMEOUT);
+    for (long long q = 0; q < kWaitLimit; ++q)
+      if (mbar_try_wait(smem_u32(mbar), (uint32_t)((issued - 1) & 1))) break;
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0) {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS));
+  }
+}
+
+int solve64_tc_chunk(const Unit* d_units, int n_units, const char* fac_base, char* ws, int nrhs, int32_t* stat,
+                     cudaStream_t st) {
+  static bool attr_set = false;
+  if (!attr_set) {
+    LSMS_CUDA_TRY(cudaFuncSetAttribute(k_solve64_tc<oz::kSolveDigits>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       oz::kSolveSmem<oz::kSolveDigits>));
+    attr_set = true;
+  }
+  LSMS_LAUNCH(k_solve64_tc<oz::kSolveDigits>, dim3(n_units, (nrhs + oz::NCC - 1) / oz::NCC), dim3(oz::NT),
+              oz::kSolveSmem<oz::kSolveDigits>, st, d_units,
+              fac_base, ws, nrhs, stat);
   return LSMS_OK;
 }
 
