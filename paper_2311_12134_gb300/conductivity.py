@@ -32,6 +32,13 @@ def check_unit_status(status):
     return st
 
 
+# Adjoint workspace when the caller gave no cap (the library's own default chunk budget).  Sized as
+# the forward's, which holds only right-hand sides when the factors are kept, the adjoint ran in
+# chunks of few units: 108 chunks and 243 ms per step for 108 atoms of n = 880 (conjugate pairs), 32
+# chunks and 17 ms for the 32-atom FP64 step; in one chunk 18.6 and 4.0 ms.
+ADJOINT_CHUNK_BYTES = 8 << 30
+
+
 class Problem:
     """One structure on one CUDA device.
 
@@ -75,6 +82,7 @@ class Problem:
         mn, al = B.tau_workspace_bytes(self.liz, self.lmax, nE, prec | self._ws_flags)
         ws = al if workspace_bytes is None else min(al, max(mn, int(workspace_bytes)))
         self.workspace = torch.empty(ws, dtype=torch.uint8, device=self.device)
+        self._capped = workspace_bytes is not None
         self.lu_store = None
         if keep_factors:
             self.lu_store = torch.empty(B.lu_store_bytes(self.liz, self.lmax, nE, prec), dtype=torch.uint8,
@@ -151,14 +159,26 @@ class Problem:
         grad_tinv_species))."""
         return _step(self, grad_sigma, tinv)
 
+    def _adjoint_workspace(self, mn, al):
+        """Workspace of the adjoint, between the sizes for one atom and for all units: as large as the
+        forward's; without a cap from the caller, up to ADJOINT_CHUNK_BYTES where the memory is there."""
+        import torch
+        small = min(al, max(mn, self.workspace.numel()))
+        size = small if self._capped else min(al, max(small, ADJOINT_CHUNK_BYTES))
+        try:
+            return torch.empty(size, dtype=torch.uint8, device=self.device)
+        except torch.OutOfMemoryError:
+            if size == small:
+                raise
+            return torch.empty(small, dtype=torch.uint8, device=self.device)
+
     def backward(self, grad_sigma, tinv=None, stream=None):
         """PyTorch gradients of Re sum(conj(grad_sigma) sigma): per site [nE, N, K, K] and per species."""
         import torch
         if self._bw_ws is None:
             mn, al = B.backward_workspace_bytes(self.liz, self.lmax, self.z.shape[0],
                                                 B._prec(self.precision, self.conj_pairs) | self._ws_flags)
-            self._bw_ws = torch.empty(min(al, max(mn, self.workspace.numel())), dtype=torch.uint8,
-                                      device=self.device)
+            self._bw_ws = self._adjoint_workspace(mn, al)
         autotune.apply(self.tuning)
         t = self.tinv if tinv is None else tinv
         out = B.kubo_sigma_backward(self.liz, self.lmax, self.species, t, self.z, self.J, self.tau, self.volume,
@@ -182,7 +202,7 @@ class Problem:
         self._maybe_check(st)
         del ws
         mn, al = B.backward_workspace_bytes(self.liz, self.lmax, nE, prec)
-        bws = torch.empty(min(al, max(mn, self.workspace.numel())), dtype=torch.uint8, device=self.device)
+        bws = self._adjoint_workspace(mn, al)
         bst = torch.empty_like(self.bw_status)
         out = B.kubo_sigma_backward(self.liz, self.lmax, self.species, tinv, self.z, self.J, tau, self.volume,
                                     grad_sigma.contiguous(), self.precision, lu_store=None, unit_status=bst,
