@@ -51,7 +51,7 @@
  * Concurrency inside a call: lsms_tau_blocks and lsms_kubo_sigma_backward split
  * each chunk of units at atom boundaries into up to four parts (option
  * "streams", else the environment variable LSMS_STREAMS, 1..4, read once;
- * default 4) that run on the caller's
+ * else 4, or 1 for small chunks) that run on the caller's
  * stream and on side streams, forked from and joined back into the caller's
  * stream by events (a capture records them as graph edges).  The side streams
  * are created by the first such call on each host thread and device.  With the
@@ -334,29 +334,26 @@ int lsms_kubo_sigma_backward(const lsms_liz* liz, int lmax, const int32_t* speci
  *   "ir_max_sweeps"   refinement sweeps of the mixed form before
  *                     LSMS_UNIT_NOCONV (default 6; 0..64)
  *   "streams"         concurrent parts per chunk (1..4; 0 = the environment
- *                     variable LSMS_STREAMS, else 4)
+ *                     variable LSMS_STREAMS, else 4, or 1 for small chunks and
+ *                     where the solves run as block steps)
  *   "residual_tc"     1 (default): the mixed form's refinement residual for 9
  *                     or more right-hand sides runs on the tensor cores (bf16
  *                     fixed-point digits, exact FP32 accumulation, about 2^-48
  *                     of |M| |X|); 0: double-float arithmetic on the FP32 pipes
- *   "solve_cols"      right-hand-side columns per CTA of the mixed form's
- *                     triangular solves above 8 columns (8, 16 or 32; 0 = 8 up to
- *                     16 columns, else 16): a tile shape the autotuner picks
- *   "solve_regs"      0 (default): 8- and 16-column solve CTAs sized for 8 CTAs
- *                     per SM (64 registers); 1: for 4 CTAs per SM (128 registers);
- *                     2: for 6 CTAs per SM (85 registers)
+ *   "solve_cols"      0, 8, 16 or 32 and
+ *   "solve_regs"      0..2: tile shapes of an earlier form of the solves; accepted
+ *                     and kept, without effect
  *   "nvtx"            1: NVTX ranges around the stages of each call (assembly +
  *                     LU, solve + refinement, traces, adjoint right-hand sides
  *                     and site products, FP64 fallback); 0 (default): none
  *   "solve_steps"     1: the mixed form's triangular solves run as one CTA
- *                     chain of block steps per unit and column slice (shaped by
- *                     solve_cols / solve_regs); 2: as one launch per 32-row block
- *                     step over all units of a chunk, the row update spread over
- *                     many CTAs on the FP32 pipes; 3: the same with the row
- *                     updates as 3xTF32 products on the tensor cores; 0
- *                     (default): block steps when a chunk part has fewer than two
- *                     chains per SM (few, large LIZ matrices; tensor cores from 9
- *                     columns), else chains
+ *                     chain per unit (row products on the tensor cores from 9
+ *                     right-hand sides); 2: as one launch per 32-row block step
+ *                     over all units of a chunk, the row update spread over many
+ *                     CTAs on the FP32 pipes; 3: the same with the row updates as
+ *                     3xTF32 products on the tensor cores; 0 (default): chains,
+ *                     but block steps (2) for few units of large matrices
+ *                     (n >= 3000 and at most n / 64 units in a chunk part)
  * LSMS_ERR_ARG for an unknown name or a value out of range. */
 int lsms_set_option(const char* name, double value);
 int lsms_get_option(const char* name, double* value);

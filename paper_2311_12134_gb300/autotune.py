@@ -4,15 +4,12 @@ The batched path has a few shapes whose best value depends on the LIZ matrix
 size n and on how many (atom, energy) units a step holds (how much parallelism
 the batched launches have):
 
-* ``solve_cols``  right-hand-side columns per CTA of the mixed form's triangular
-                  solves (8, 16 or 32): wider slices read the factors fewer
-                  times, narrower slices run more independent block-step chains;
-* ``solve_regs``  8 solve CTAs per SM with 64 registers (0), 4 with 128 (1) or
-                  6 with 85 (2);
-* ``solve_steps`` the solves by the library's choice (0), as one CTA chain per
-                  unit and slice (1) or as one launch per block step over all
-                  units, row updates on the FP32 pipes (2) or the tensor cores (3);
-* ``streams``     concurrent parts of each chunk of units (2 or 4).
+* ``solve_steps`` the mixed form's triangular solves by the library's choice (0), as one CTA
+                  chain per unit (1) or as one launch per block step over all units, row
+                  updates on the FP32 pipes (2) or the tensor cores (3);
+* ``streams``     concurrent parts of each chunk of units (2 or 4; 0: the library's choice);
+* ``solve_cols``, ``solve_regs``  shapes of an earlier form of the solves, without effect now
+                  (kept in the settings: the library accepts them).
 
 ``tune`` times ``Problem.step`` (forward + adjoint) under every candidate with
 CUDA events and keeps the fastest; the results live in a JSON table keyed by
@@ -39,18 +36,12 @@ TABLE = os.path.join(HERE, "tuning_gb300.json")
 N_BUCKETS = (256, 512, 768, 1024, 1536, 2048, 3072, 4096, 8192, 16384)
 U_BUCKETS = (1024, 8192, 65536, 1 << 30)
 
-DEFAULTS = {"solve_cols": 0, "solve_regs": 0, "solve_steps": 0, "streams": 4}
+DEFAULTS = {"solve_cols": 0, "solve_regs": 0, "solve_steps": 0, "streams": 0}
 
 
 def candidates():
-    out = []
-    for streams in (2, 4):
-        out.append({"solve_cols": 0, "solve_regs": 0, "solve_steps": 0, "streams": streams})
-        out.append({"solve_cols": 0, "solve_regs": 0, "solve_steps": 2, "streams": streams})
-        out.append({"solve_cols": 0, "solve_regs": 0, "solve_steps": 3, "streams": streams})
-        for cols, regs in ((0, 0), (0, 1), (0, 2), (8, 0), (8, 1), (8, 2), (16, 0), (16, 1), (16, 2), (32, 0)):
-            out.append({"solve_cols": cols, "solve_regs": regs, "solve_steps": 1, "streams": streams})
-    return out
+    return [{"solve_cols": 0, "solve_regs": 0, "solve_steps": steps, "streams": streams}
+            for streams in (0, 2, 4) for steps in (0, 1, 2, 3)]
 
 
 def size_class(gpu_name, precision, lmax, n_max, n_units):

@@ -92,11 +92,11 @@ constexpr double kIrTol = 1e-10;
 static std::atomic<double> g_opt_growth_limit{1e3};
 static std::atomic<int> g_opt_fallback_slots{8};
 static std::atomic<int> g_opt_ir_max_sweeps{kIrMaxIter};
-static std::atomic<int> g_opt_streams{0};  // 0: LSMS_STREAMS or the default
+static std::atomic<int> g_opt_streams{0};  // 0: LSMS_STREAMS, else by the chunk's size (parts_of)
 static std::atomic<int> g_opt_residual_tc{1};
-static std::atomic<int> g_opt_solve_cols{0};  // 0: 8 columns per CTA up to 16 right-hand sides, else 16
+static std::atomic<int> g_opt_solve_cols{0};  // accepted and kept; the solves have one shape
 static std::atomic<int> g_opt_solve_regs{0};
-static std::atomic<int> g_opt_solve_steps{0};  // 0, 1: one CTA chain per unit and slice; 2: block-step launches
+static std::atomic<int> g_opt_solve_steps{0};  // 0: by size (solve_path); 1: one CTA chain per unit; 2, 3: block-step launches
 static std::atomic<int> g_opt_nvtx{0};
 
 // NVTX range over one stage of a call (option "nvtx"; the header-only NVTX3
@@ -112,8 +112,6 @@ struct NvtxRange {
   }
 };
 int opt_residual_tc() { return g_opt_residual_tc.load(); }
-int opt_solve_cols() { return g_opt_solve_cols.load(); }
-int opt_solve_regs() { return g_opt_solve_regs.load(); }
 int opt_solve_steps() { return g_opt_solve_steps.load(); }
 double opt_growth_limit() { return g_opt_growth_limit.load(); }
 int opt_fallback_slots() { return g_opt_fallback_slots.load(); }
@@ -1652,16 +1650,33 @@ struct SideStreams {
   cudaEvent_t fork = nullptr, join[kMaxParts - 1] = {};
 };
 
-// Number of concurrent parts per chunk: the "streams" option if set, else the
-// environment variable LSMS_STREAMS (1..4, read once), else 4.
-static int stream_parts() {
+// Concurrent parts asked for: the "streams" option if set, else the environment variable
+// LSMS_STREAMS (1..4, read once), else 0 (parts_of decides).
+static int asked_parts() {
   static const int env_parts = [] {
     const char* e = std::getenv("LSMS_STREAMS");
-    const int v = e ? std::atoi(e) : 4;
-    return std::min(std::max(v, 1), kMaxParts);
+    return e ? std::min(std::max(std::atoi(e), 1), kMaxParts) : 0;
   }();
   const int o = g_opt_streams.load();
   return o > 0 ? std::min(o, kMaxParts) : env_parts;
+}
+
+// Parts of a chunk.  By default four, but one
+//  - for a small chunk (rows of all its factored matrices below 64k), whose launches are mostly
+//    latency: 64 units of n = 208 took 2.54 ms per step in one part, 3.27 in four; 108 of n = 243
+//    3.16 and 3.67; from 216 units of n = 880 on four parts gain (18.7 and 17.8 ms);
+//  - where the solves run as block-step launches: a part's thousands of launches fill the launch
+//    queue before the next part's first one is enqueued, so parts run one after the other, each on a
+//    nearly idle GPU (54 atoms of n = 2192 90 ms in one part, 155 in four; 2 of n = 15,440 970 and
+//    1296 in two).
+static int parts_of(const Plan& p, const Chunk& ch) {
+  const int asked = asked_parts();
+  if (asked) return asked;
+  int64_t rows = 0;
+  for (int f = ch.f0; f < ch.f1; ++f) rows += p.fac_units[f].n;
+  if (rows < 65536) return 1;
+  if (p.precision == LSMS_MIXED && solve_path(ch.u1 - ch.u0, ch.n_max) != 1) return 1;
+  return kMaxParts;
 }
 
 static int side_streams(SideStreams** out) {
@@ -1706,7 +1721,7 @@ static int split_chunk(const Plan& p, const Chunk& ch, int want, Chunk* part) {
 template <typename F>
 static int run_split(const Call& c, const Plan& p, const Chunk& ch, F run) {
   Chunk part[kMaxParts];
-  const int np = g_timer_on.load(std::memory_order_relaxed) ? 1 : split_chunk(p, ch, stream_parts(), part);
+  const int np = g_timer_on.load(std::memory_order_relaxed) ? 1 : split_chunk(p, ch, parts_of(p, ch), part);
   if (np == 1) return run(ch, c.st);
   SideStreams* ss = nullptr;
   int rc = side_streams(&ss);
@@ -1785,7 +1800,7 @@ extern "C" int lsms_get_option(const char* name, double* value) {
   if (n == "growth_limit") *value = g_opt_growth_limit.load();
   else if (n == "fallback_slots") *value = g_opt_fallback_slots.load();
   else if (n == "ir_max_sweeps") *value = g_opt_ir_max_sweeps.load();
-  else if (n == "streams") *value = stream_parts();
+  else if (n == "streams") *value = asked_parts() ? asked_parts() : kMaxParts;
   else if (n == "residual_tc") *value = g_opt_residual_tc.load();
   else if (n == "solve_cols") *value = g_opt_solve_cols.load();
   else if (n == "solve_regs") *value = g_opt_solve_regs.load();

@@ -247,10 +247,13 @@ enum RhsField { RHS_X = 0, RHS_X32 = 1 };
 int residual_tc_chunk(const Unit* d_units, int n_units, int n_max, const char* fac_base, char* ws, int K, int nrhs,
                       bool explicit_b, const int32_t* done, int32_t* stat, cudaStream_t st);
 int opt_residual_tc();
-int opt_solve_cols();
-int opt_solve_regs();
 int opt_solve_steps();
+int solve_path(int n_units, int n_max);  // 1: chains, 2 or 3: block-step launches (lu.cu)
 
+// The complex64 solves L U X = X (permuted) on the X32 field with 9 to 32 right-hand sides, one chain
+// per unit with the row products on the tensor cores (tc_solve.cu).
+int solve_tc_chunk(const Unit* d_units, int n_units, const char* fac_base, char* ws, int nrhs, const int32_t* done,
+                   int32_t* stat, cudaStream_t st);
 // One block step of the complex64 triangular solves on the tensor cores (tc_gemm.cu):
 // forward X[rows >= 32 (s + 1)] -= L[., block s] X[block s], backward
 // X[rows < 32 s] -= U[., block s] X[block s], on the X32 field, nrhs <= 32.

@@ -622,45 +622,28 @@ __global__ void __launch_bounds__(256) k_swap_trsm(const Unit* __restrict__ unit
 }
 
 // ------------------------------------------------------------------ complex64 solve
-// The complex64 solve of the mixed form, specialised on the padded right-hand-side
-// count NCOL (columns >= nrhs are zero and never stored).  The update of the rows
-// below (forward) or above (backward) a solved block gives each thread one row
-// and G = min(NCOL, 8) columns: per step j one coalesced 8-byte load of the
-// factor, G/2 16-byte shared-memory loads of the solved block and 4 G FMAs.
+// The complex64 solve of the mixed form with at most 8 right-hand sides, specialised on
+// the padded column count NCOL (columns >= nrhs are zero and never stored).  The update
+// of the rows below (forward) or above (backward) a solved block gives each thread one
+// row: per step j one coalesced 8-byte load of the factor, NCOL / 2 16-byte
+// shared-memory loads of the solved block and 4 NCOL FMAs.
 constexpr int kSolveThreads = 256;  // complex64 solve CTA
 
 template <int NCOL, int NT>
 __device__ __forceinline__ void update_rows_c64(const float2* __restrict__ A, float2* X, const float2 (*sX)[NCOL],
                                                 int n, int k, int nbp, int r0, int r1, int nrhs, int tid) {
-  constexpr int G = NCOL < 8 ? NCOL : 8;
-  constexpr int NG = NCOL / G;
   constexpr int NB = 32;
-  const int rows = r1 - r0;
-  if (rows <= 0) return;
-  // work item = (row, group of G columns); a warp takes 32 consecutive rows of one
-  // group and the NG groups of the same rows go to consecutive warps, so the
-  // factor's 32-row segments are fetched once and reused from L1 by the others
-  const int chunks = (rows + 31) / 32;
-  for (int idx = tid; idx < chunks * 32 * NG; idx += NT) {
-    const int gi = (idx >> 5) % NG;
-    const int i = r0 + ((idx >> 5) / NG) * 32 + (idx & 31);
-    if (i >= r1) continue;
-    const int g = gi * G;
+  for (int i = r0 + tid; i < r1; i += NT) {
     // the factor entries of this thread's next item (read once from DRAM) are
-    // requested into L2 now, by the warps of the first column group only (with
-    // 32 columns the extra L2 traffic cost more than the latency it hid)
-    if constexpr (NCOL <= 16) {
-      const int nidx = idx + NT;
-      const int ni = r0 + ((nidx >> 5) / NG) * 32 + (nidx & 31);
-      if (gi == 0 && ni < r1 && (nidx >> 5) % NG == 0) {
-        const float2* An = A + (size_t)k * n + ni;
+    // requested into L2 now
+    if (i + NT < r1) {
+      const float2* An = A + (size_t)k * n + i + NT;
 #pragma unroll 4
-        for (int j = 0; j < nbp; ++j) asm volatile("prefetch.global.L2 [%0];" ::"l"(An + (size_t)j * n));
-      }
+      for (int j = 0; j < nbp; ++j) asm volatile("prefetch.global.L2 [%0];" ::"l"(An + (size_t)j * n));
     }
-    float2 acc[G];
+    float2 acc[NCOL];
 #pragma unroll
-    for (int c = 0; c < G; ++c) acc[c] = (g + c < nrhs) ? X[(size_t)(g + c) * n + i] : make_float2(0.f, 0.f);
+    for (int c = 0; c < NCOL; ++c) acc[c] = (c < nrhs) ? X[(size_t)c * n + i] : make_float2(0.f, 0.f);
     const float2* Ai = A + (size_t)k * n + i;
     if (nbp == NB) {
 #pragma unroll 1
@@ -671,8 +654,8 @@ __device__ __forceinline__ void update_rows_c64(const float2* __restrict__ A, fl
 #pragma unroll
         for (int jj = 0; jj < 8; ++jj) {
 #pragma unroll
-          for (int c = 0; c < G; c += 2) {
-            const float4 xx = *reinterpret_cast<const float4*>(&sX[j0 + jj][g + c]);
+          for (int c = 0; c < NCOL; c += 2) {
+            const float4 xx = *reinterpret_cast<const float4*>(&sX[j0 + jj][c]);
             acc[c] = cfms(l[jj], make_float2(xx.x, xx.y), acc[c]);
             acc[c + 1] = cfms(l[jj], make_float2(xx.z, xx.w), acc[c + 1]);
           }
@@ -682,16 +665,16 @@ __device__ __forceinline__ void update_rows_c64(const float2* __restrict__ A, fl
       for (int j = 0; j < nbp; ++j) {
         const float2 l = Ai[(size_t)j * n];
 #pragma unroll
-        for (int c = 0; c < G; c += 2) {
-          const float4 xx = *reinterpret_cast<const float4*>(&sX[j][g + c]);
+        for (int c = 0; c < NCOL; c += 2) {
+          const float4 xx = *reinterpret_cast<const float4*>(&sX[j][c]);
           acc[c] = cfms(l, make_float2(xx.x, xx.y), acc[c]);
           acc[c + 1] = cfms(l, make_float2(xx.z, xx.w), acc[c + 1]);
         }
       }
     }
 #pragma unroll
-    for (int c = 0; c < G; ++c)
-      if (g + c < nrhs) X[(size_t)(g + c) * n + i] = acc[c];
+    for (int c = 0; c < NCOL; ++c)
+      if (c < nrhs) X[(size_t)c * n + i] = acc[c];
   }
 }
 
@@ -866,28 +849,24 @@ __global__ void __launch_bounds__(256) k_perm_rows(const Unit* __restrict__ unit
   for (int r = threadIdx.x; r < n; r += blockDim.x) X[r] = sv[r];
 }
 
-// One CTA of NT threads per unit and slice of NCOL right-hand-side columns
-// (blockIdx.y; several CTAs resident per SM, so one chain's block phases overlap
-// the others' row updates): L y = P b (unit lower, L in the row order of P, the
-// right-hand sides permuted by k_perm_rows before), then U x = y, on the
-// n x nrhs column-major block X.  Each 32-row block step multiplies its rows by
+// Up to 8 right-hand sides: one CTA per unit (several resident per SM, so one chain's
+// block phases overlap the others' row updates): L y = P b (unit lower, L in the row
+// order of P, the right-hand sides permuted by k_perm_rows before), then U x = y, on
+// the n x nrhs column-major block X.  Each 32-row block step multiplies its rows by
 // the stored inverse of the diagonal block (all threads, no serial chain) and
 // updates the rows below (above, going back) with the block's 32 columns of L (U).
-template <int NCOL, int NT, int MINB = 1024 / NT>
-__global__ void __launch_bounds__(NT, MINB) k_solve_c64(const Unit* __restrict__ units, const char* fac_base,
-                                                     char* ws, int which, int nrhs, const int32_t* done) {
-  static_assert(NCOL >= 2 && NCOL % 2 == 0 && NCOL <= 32, "padded column count");
+template <int NCOL>
+__global__ void __launch_bounds__(kSolveThreads, 4) k_solve_c64(const Unit* __restrict__ units, const char* fac_base,
+                                                                char* ws, int nrhs, const int32_t* done) {
+  static_assert(NCOL >= 2 && NCOL % 2 == 0 && NCOL <= 8, "padded column count");
+  constexpr int NT = kSolveThreads;
   constexpr int NB = kDiagNB;
   const Unit u = units[blockIdx.x];
   if (done && done[u.stat_off]) return;
   const int n = u.n;
-  // columns [NCOL y, NCOL y + NCOL) of the right-hand sides (slice y = blockIdx.y)
-  const int c_off = blockIdx.y * NCOL;
-  nrhs = min(NCOL, nrhs - c_off);
-  if (nrhs <= 0) return;
   const float2* A = reinterpret_cast<const float2*>(fac_base + u.fac_off);
   const float2* D = reinterpret_cast<const float2*>(fac_base + u.m64_off + diag_inv_rel_off(n));
-  float2* X = reinterpret_cast<float2*>(ws + (which == RHS_X ? u.x_off : u.x32_off)) + (size_t)c_off * n;
+  float2* X = reinterpret_cast<float2*>(ws + u.x32_off);
   __shared__ float2 sT[NB][NB + 1];                 // inverse of the diagonal block
   __shared__ __align__(16) float2 sX[NB][NCOL];     // the block's solved rows
   __shared__ float2 sIn[NB][NCOL + 1];              // the block's rows before the inverse
@@ -1229,6 +1208,17 @@ static int solve_steps_tc(const Unit* d_units, int n_units, int n_max, const cha
   return LSMS_OK;
 }
 
+// Option "solve_steps": 1 = one CTA chain per unit; 2 = block-step launches (row updates on the FP32
+// pipes); 3 = the same on the tensor cores; 0 (default) = chains, but block steps for few units of
+// large matrices, which leave most SMs idle: a chain's time grows with n^2, that of the 2 n / 32
+// launches with n and the units.  Measured, solves of one forward (chains / steps): n = 2192, 4 units
+// 26.4 / 29.0 ms, 32 units 26.9 / 34.2; n = 4144, 4 units 47.4 / 29.2, 32 units 47.7 / 36.6;
+// n = 8496, 4 units 240 / 67.
+int solve_path(int n_units, int n_max) {
+  const int o = opt_solve_steps();
+  return o ? o : (n_max >= 3000 && n_units <= n_max / 64 ? 2 : 1);
+}
+
 template <typename R>
 int lu_solve_chunk(const Unit* d_units, int n_units, int n_max, const char* fac_base, char* ws, int which_rhs,
                    int nrhs, const int32_t* done, int32_t* stat, cudaStream_t st) {
@@ -1245,58 +1235,19 @@ int lu_solve_chunk(const Unit* d_units, int n_units, int n_max, const char* fac_
       perm_attr = pb;
     }
     LSMS_LAUNCH(k_perm_rows, dim3(nrhs, n_units), dim3(256), pb, st, d_units, fac_base, ws, nrhs, done);
-    // option "solve_steps": 1 = one CTA chain per unit and column slice; 2 = block-step launches
-    // (row updates on the FP32 pipes); 3 = block-step launches with the row updates on the tensor
-    // cores; 0 (default) = block steps when the chains could not fill the GPU (fewer than two per
-    // SM: few units of large LIZ matrices), on the tensor cores from 9 columns, else chains
-    int steps = opt_solve_steps();
-    if (steps == 0) {
-      static int sms = 0;
-      if (!sms) {
-        int dev = 0;
-        LSMS_CUDA_TRY(cudaGetDevice(&dev));
-        LSMS_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-      }
-      const int slices = nrhs <= 16 ? 1 : 2;
-      steps = (long long)n_units * slices < 2LL * sms ? (nrhs > 8 ? 3 : 2) : 1;
-    }
+    const int steps = solve_path(n_units, n_max);
     if (steps == 3) return solve_steps_tc(d_units, n_units, n_max, fac_base, ws, nrhs, done, stat, st);
     if (steps == 2) {
       if (nrhs <= 8) return solve_steps<8>(d_units, n_units, n_max, fac_base, ws, nrhs, done, st);
       if (nrhs <= 16) return solve_steps<16>(d_units, n_units, n_max, fac_base, ws, nrhs, done, st);
       return solve_steps<32>(d_units, n_units, n_max, fac_base, ws, nrhs, done, st);
     }
-    // more than 8 columns: column slices per CTA (option "solve_cols"; default 8
-    // for up to 16 columns, 16 above), each slice a CTA with its own chain of
-    // block steps; wider slices read the factors fewer times, narrower ones give
-    // more concurrent chains
+    // one chain per unit: from 9 columns on the tensor cores (tc_solve.cu), below in FP32
+    if (nrhs > 8) return solve_tc_chunk(d_units, n_units, fac_base, ws, nrhs, done, stat, st);
     const dim3 g1(n_units), b256(kSolveThreads);
-    if (nrhs <= 2) LSMS_LAUNCH((k_solve_c64<2, kSolveThreads>), g1, b256, 0, st, d_units, fac_base, ws, which_rhs, nrhs, done);
-    else if (nrhs <= 4) LSMS_LAUNCH((k_solve_c64<4, kSolveThreads>), g1, b256, 0, st, d_units, fac_base, ws, which_rhs, nrhs, done);
-    else if (nrhs <= 8) LSMS_LAUNCH((k_solve_c64<8, kSolveThreads>), g1, b256, 0, st, d_units, fac_base, ws, which_rhs, nrhs, done);
-    else {
-      // option "solve_regs": 0 = 8 CTAs of 128 threads per SM (64 registers), 1 = 4 (128 registers),
-      // 2 = 6 (85 registers)
-      int sl = opt_solve_cols();
-      if (sl <= 0) sl = nrhs <= 16 ? 8 : 16;
-      if (sl == 32 && nrhs <= 16) sl = 16;  // one slice holds every column
-      const int regs = opt_solve_regs();
-      const dim3 gs(n_units, (nrhs + sl - 1) / sl);
-#define LSMS_SOLVE(NCOL, NT, MINB) \
-  LSMS_LAUNCH((k_solve_c64<NCOL, NT, MINB>), gs, dim3(NT), 0, st, d_units, fac_base, ws, which_rhs, nrhs, done)
-      if (sl == 8) {
-        if (regs == 2) LSMS_SOLVE(8, 128, 6);
-        else if (regs) LSMS_SOLVE(8, 128, 4);
-        else LSMS_SOLVE(8, 128, 8);
-      } else if (sl == 16) {
-        if (regs == 2) LSMS_SOLVE(16, 128, 6);
-        else if (regs) LSMS_SOLVE(16, 128, 4);
-        else LSMS_SOLVE(16, 128, 8);
-      } else {
-        LSMS_SOLVE(32, 256, 2);
-      }
-#undef LSMS_SOLVE
-    }
+    if (nrhs <= 2) LSMS_LAUNCH(k_solve_c64<2>, g1, b256, 0, st, d_units, fac_base, ws, nrhs, done);
+    else if (nrhs <= 4) LSMS_LAUNCH(k_solve_c64<4>, g1, b256, 0, st, d_units, fac_base, ws, nrhs, done);
+    else LSMS_LAUNCH(k_solve_c64<8>, g1, b256, 0, st, d_units, fac_base, ws, nrhs, done);
   } else {
     return solve64_tc_chunk(d_units, n_units, fac_base, ws, nrhs, stat, st);
   }
