@@ -26,14 +26,19 @@
 //                one element of X into the six planes of B (no-swizzle K-major
 //                core-matrix layout in shared memory), real and imaginary
 //                parts in the two lanes of the paired FP32 instructions;
-//   one thread   issues the 42 tcgen05.mma (M = 128, N = 32, K = 16) of the
-//                chunk and commits them to an mbarrier (bounded waits, polled
-//                by one warp);
+//   one thread   issues the 12 tcgen05.mma of the chunk (one per digit of M and
+//                16 K, N = 32 times the digits of X it meets) and commits them
+//                to an mbarrier (bounded waits, polled by one warp);
 //   every 4th    warps 0-3 add the real outputs of their TMEM lanes, warps 4-7
 //                the imaginary ones.
+// Bound by the instructions of the splitting (issue slots half used, tensor pipe
+// 20 %), with both CTAs of an SM in it at once part of the time.  Measured (1,488 units of
+// n about 850, 16 and 32 columns): 17.0 ms, against 22.7 ms with one instruction
+// per digit pair, a rounding and two multiplications per digit and stores of B
+// that met in the same banks.  One CTA of 512 threads per SM with two operand
+// stages took 22.9 ms, with cp.async copies of M three chunks ahead 28.4; the
+// lines of M requested into L2 two chunks ahead 20.4 (the loads are not what waits).
 #include <cstdint>
-
-#include <cuda_bf16.h>
 
 #include "common.cuh"
 
@@ -138,44 +143,36 @@ __device__ __forceinline__ float2 rint2(float2 x) {
   return __fadd2_rn(__fadd2_rn(x, big), nbig);
 }
 
-// (r, c) <- (r + c, rounding error) exactly (two-sum), lane-wise.
-__device__ __forceinline__ void two_sum2(float2& r, float2& c) {
-  const float2 a = __fadd2_rn(r, c);
-  const float2 bb = __fadd2_rn(a, make_float2(-r.x, -r.y));
-  const float2 e = __fadd2_rn(__fadd2_rn(r, make_float2(bb.x - a.x, bb.y - a.y)), __fadd2_rn(c, make_float2(-bb.x, -bb.y)));
-  r = a;
-  c = e;
-}
-
-// The six digits of the double-float value (h + l) 2^7 / 2^E, sc = 2^{7 - E},
-// two values at once (lanes).  With r the remainder in units of the next digit:
-// d = rint(r), r = 256 (r - d) (exact); the low part c (|c| <= 2^-17 at the
-// start) is folded in exactly (two-sum) before digits 3 and 5, when two steps of
-// 256 have made it as large as half a unit, so every digit satisfies |d| <= 129.
+// The six digits of the double-float value (h + l) 2^7 / 2^E, sc = 2^{7 - E}, two values at
+// once (lanes): digit 1, then digits 2, 3 and 4, 5 as 16-bit integers q that split into
+// rint(q / 256) and the rest, then digit 6.  Every remainder is exact; the low part
+// c = l sc (at most 2^-17) enters q of digits 4, 5 and the remainder after it, so those
+// two digits may reach 192 and 129, the others 128.
 __device__ __forceinline__ void digits6x2(float2 h, float2 l, float2 sc, float2* d) {
-  const float2 k256 = make_float2(256.f, 256.f), nk256 = make_float2(-256.f, -256.f);
-  const float2 k64k = make_float2(65536.f, 65536.f);
-  float2 r = __fmul2_rn(h, sc), c = __fmul2_rn(l, sc);
-#pragma unroll
-  for (int s = 0; s < ND; ++s) {
-    if (s == 2 || s == 4) {
-      c = __fmul2_rn(c, k64k);
-      two_sum2(r, c);
-    }
-    const float2 q = rint2(r);
-    d[s] = q;
-    if (s + 1 < ND) r = __ffma2_rn(q, nk256, __fmul2_rn(r, k256));  // 256 r - 256 q: exact
-  }
+  const float2 m1 = make_float2(-1.f, -1.f), k64k = make_float2(65536.f, 65536.f);
+  const float2 k32 = make_float2(4294967296.f, 4294967296.f);
+  const float2 i256 = make_float2(0.00390625f, 0.00390625f), k256 = make_float2(256.f, 256.f),
+               n256 = make_float2(-256.f, -256.f);
+  const float2 big = make_float2(12582912.f, 12582912.f), nbig = make_float2(-12582912.f, -12582912.f);
+  const float2 x = __fmul2_rn(h, sc), c = __fmul2_rn(l, sc);
+  d[0] = rint2(x);
+  const float2 r = __fmul2_rn(__ffma2_rn(d[0], m1, x), k64k);
+  const float2 q = rint2(r);
+  d[1] = __fadd2_rn(__ffma2_rn(q, i256, big), nbig);
+  d[2] = __ffma2_rn(d[1], n256, q);
+  const float2 e = __fmul2_rn(__ffma2_rn(q, m1, r), k64k);
+  const float2 q2 = rint2(__ffma2_rn(c, k32, e));
+  d[3] = __fadd2_rn(__ffma2_rn(q2, i256, big), nbig);
+  d[4] = __ffma2_rn(d[3], n256, q2);
+  const float2 f = __ffma2_rn(c, k32, __ffma2_rn(q2, m1, e));
+  d[5] = __fadd2_rn(__ffma2_rn(f, k256, big), nbig);
 }
 
+// bf16 values of small integers: the upper halves of their FP32 bits, exactly
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);  // digits are small integers: exact
-  return *reinterpret_cast<const uint32_t*>(&v);
+  return __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x7632);
 }
-__device__ __forceinline__ unsigned short bf16_bits(float x) {
-  const __nv_bfloat16 v = __float2bfloat16_rn(x);
-  return *reinterpret_cast<const unsigned short*>(&v);
-}
+__device__ __forceinline__ unsigned short bf16_bits(float x) { return (unsigned short)(__float_as_uint(x) >> 16); }
 
 }  // namespace rtc
 
@@ -231,8 +228,9 @@ __global__ void __launch_bounds__(256, 2) k_residual_tc(const Unit* __restrict__
   const bool alive = arow < n;
   const int EA = alive ? scale_exp(rowmax[arow]) : 0;
   const float2 rsc = make_float2(pow2f(7 - EA), pow2f(7 - EA));
-  // B: element (row j, column cc) of the chunk's 16 x 16 block of X
-  const int bcc = tid & 15, bj = tid >> 4;
+  // B: element (row j, column cc) of the chunk's 16 x 16 block of X; a warp's 8 columns x 4 rows
+  // store to 16 words of different banks
+  const int bcc = (tid & 7) + 8 * (warp & 1), bj = ((tid >> 3) & 3) + 4 * (warp >> 1);
   const int bcol = col0 + bcc;
   const int F_b = bcol < nrhs ? scale_exp(colmax[bcol]) : 0;
   const float2 csc = make_float2(pow2f(7 - F_b), pow2f(7 - F_b));
@@ -269,8 +267,10 @@ __global__ void __launch_bounds__(256, 2) k_residual_tc(const Unit* __restrict__
   };
   auto flush = [&](uint32_t tmem) {
     const uint32_t base = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(half * NC);
+    // classes 0..3 by two-sum; the last two (below 2^-9 of a unit of class 0, as large as the
+    // rounding errors that acct collects) go straight into acct
 #pragma unroll 1
-    for (int g = 0; g < NG; ++g) {
+    for (int g = 0; g < 4; ++g) {
       float v[16];
       tmem_ld16(base + (uint32_t)(g * NOUT), v);
       const float w = pow2f(-8 * g);
@@ -283,6 +283,11 @@ __global__ void __launch_bounds__(256, 2) k_residual_tc(const Unit* __restrict__
         accs[c] = a;
       }
     }
+    float v4[16], v5[16];
+    tmem_ld16(base + (uint32_t)(4 * NOUT), v4);
+    tmem_ld16(base + (uint32_t)(5 * NOUT), v5);
+#pragma unroll
+    for (int c = 0; c < NC; ++c) acct[c] += fmaf(v5[c], 0x1p-40f, v4[c] * 0x1p-32f);
   };
 
   const int nchunks = (n + KCC - 1) / KCC;
@@ -345,22 +350,18 @@ __global__ void __launch_bounds__(256, 2) k_residual_tc(const Unit* __restrict__
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     tmem = *tslot;
     if (tid == 0) {
-      const uint32_t idesc = make_idesc(TM, NOUT);
       const uint32_t a0 = smem_u32(sA), b0 = smem_u32(sB);
-      // first chunk of a window: each class starts from zero with its first product, which in
-      // this order (A digit s outer, B digit t inner) is the pair (s = 0, t = g), K step 0
+      // B's planes lie one after the other, so one instruction per digit s of A multiplies it with
+      // the digits t = 0 .. ND - 1 - s at once, into the classes g = s + t from class s on (A is read
+      // 6 times per 16 K instead of 21).  First chunk of a window: the first instruction (s = 0,
+      // every class) starts from zero.
       const bool fresh = (ch % FLUSH) == 0;
 #pragma unroll
-      for (int s = 0; s < ND; ++s) {
+      for (int ks = 0; ks < 2; ++ks)
 #pragma unroll
-        for (int t = 0; t < ND - s; ++t) {
-          const int g = s + t;  // weight class of digits (s + 1, t + 1)
-#pragma unroll
-          for (int ks = 0; ks < 2; ++ks)
-            mma_bf16(tmem + (uint32_t)(g * NOUT), make_desc(a0 + s * PLANE_A + ks * 2 * LBO),
-                     make_desc(b0 + t * PLANE_B + ks * 2 * LBO), idesc, (fresh && ks == 0 && s == 0) ? 0u : 1u);
-        }
-      }
+        for (int s = 0; s < ND; ++s)
+          mma_bf16(tmem + (uint32_t)(s * NOUT), make_desc(a0 + s * PLANE_A + ks * 2 * LBO), make_desc(b0 + ks * 2 * LBO),
+                   make_idesc(TM, NOUT * (ND - s)), (fresh && ks == 0 && s == 0) ? 0u : 1u);
       asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                        smem_u32(mbar))
                    : "memory");
