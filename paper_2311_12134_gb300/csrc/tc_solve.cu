@@ -337,6 +337,7 @@ __global__ void __launch_bounds__(ts::NT, 2) k_solve_tc(const Unit* __restrict__
                        : "memory");
         }
     };
+    // copy groups: the first two inverses and the blocks of step 0, then those of steps 1 and 2
     load_d(0);
     load_d(1);
     {
@@ -344,11 +345,17 @@ __global__ void __launch_bounds__(ts::NT, 2) k_solve_tc(const Unit* __restrict__
 #pragma unroll
       for (int i = 0; i < 3; ++i) {
         const int R = 96 - 32 * i, b = fwd ? i : 3 - i, rs = fwd ? 32 * (b + 1) : 0;
-        for (int idx = tid; idx < R * NB; idx += NT) {
+#pragma unroll 4
+        for (int q = 0; q < R * NB / NT; ++q) {
+          const int idx = tid + q * NT;
           const int r = rs + idx % R, c = 32 * b + idx / R;
-          sL[off + idx] = (r < rows && c < rows) ? __ldg(&F[(size_t)(g0 + c) * n + g0 + r]) : make_float2(0.f, 0.f);
+          const bool in = r < rows && c < rows;
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(smem_u32(sL + off + idx)),
+                       "l"(F + (in ? (size_t)(g0 + c) * n + g0 + r : 0)), "r"(in ? 8 : 0)
+                       : "memory");
         }
         off += R * NB;
+        asm volatile("cp.async.commit_group;" ::: "memory");
       }
     }
     // x = b - acc
@@ -361,13 +368,16 @@ __global__ void __launch_bounds__(ts::NT, 2) k_solve_tc(const Unit* __restrict__
       }
       sX[er * LDX + ec + c] = x;
     }
-    asm volatile("cp.async.wait_all;" ::: "memory");
+    asm volatile("cp.async.wait_group 2;" ::: "memory");
     __syncthreads();
     int off = 0;
 #pragma unroll 1
     for (int i = 0; i < 4; ++i) {
       const int b = fwd ? i : 3 - i, R = 96 - 32 * i, rs = fwd ? 32 * (b + 1) : 0;
-      if (i == 1 || i == 2) load_d(i + 1);  // its slot was last read in step i - 1
+      if (i == 1 || i == 2) {
+        load_d(i + 1);  // its slot was last read in step i - 1
+        asm volatile("cp.async.commit_group;" ::: "memory");
+      }
       prefetch(len + i + kAhead);
       if (32 * b < rows) {  // a block of the last, partial group may be missing
         // y = T^{-1} x: lane = row, warp = NCOL / 8 columns
@@ -433,7 +443,9 @@ __global__ void __launch_bounds__(ts::NT, 2) k_solve_tc(const Unit* __restrict__
         }
       }
       off += R * NB;
-      asm volatile("cp.async.wait_all;" ::: "memory");
+      // step 1 needs the second group, the later steps everything issued
+      if (i == 0) asm volatile("cp.async.wait_group 1;" ::: "memory");
+      else asm volatile("cp.async.wait_group 0;" ::: "memory");
       __syncthreads();  // the next inverse is there, this one's slot free; after the last step X is current
     }
   }
