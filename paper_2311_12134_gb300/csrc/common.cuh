@@ -123,9 +123,32 @@ __device__ __forceinline__ void df_mac(float& s, float& t, float ah, float al, f
   t += e;
 }
 
+// hi = a rounded to FP32, lo = a - hi rounded to FP32.  In the range where both parts are normal
+// floats (2^-74 <= |a| < 2^127, and zero) from the bits of a, with integer instructions: the four
+// conversions and subtractions of the plain form run on the FP64 pipe (2 lanes per SM and clock),
+// which cost the trace kernel as much as its products.  Same values as the plain form.
+__device__ __forceinline__ float2 df_split(double a) {
+  const uint32_t hw = (uint32_t)__double2hiint(a), lw = (uint32_t)__double2loint(a);
+  const uint32_t e = (hw >> 20) & 0x7ff;
+  if (e - 949u < 201u || ((hw << 1) | lw) == 0u) {
+    uint32_t top = __funnelshift_l(lw, (hw & 0xfffff) | 0x100000, 3);  // the 24 leading bits
+    int rem = (int)(lw & 0x1fffffff);                                   // the 29 others
+    if (rem > 0x10000000 || (rem == 0x10000000 && (top & 1))) {         // to nearest, ties to even
+      ++top;
+      rem -= 0x20000000;
+    }
+    const uint32_t sign = hw & 0x80000000u;
+    const uint32_t hi = (((e - 896u) << 23) + (top - 0x800000u)) | sign;
+    const float lo = (float)rem * __uint_as_float(((e - 948u) << 23) | sign);  // exponent e - 1075 + 127
+    const bool zero = e == 0u;
+    return make_float2(zero ? __uint_as_float(sign) : __uint_as_float(hi), zero ? 0.f : lo);
+  }
+  const float h = (float)a;
+  return make_float2(h, (float)(a - (double)h));
+}
 __device__ __forceinline__ float4 df_split(double2 a) {
-  const float rh = (float)a.x, ih = (float)a.y;
-  return make_float4(rh, (float)(a.x - (double)rh), ih, (float)(a.y - (double)ih));
+  const float2 re = df_split(a.x), im = df_split(a.y);
+  return make_float4(re.x, re.y, im.x, im.y);
 }
 
 __device__ __forceinline__ double2 df_join(float4 a) {
@@ -182,10 +205,7 @@ __device__ __forceinline__ float4 df_value(const DfAcc& a) {
 }
 
 // Real double-float values (hi, lo) as float2, normalised (|lo| <= ulp(hi) / 2).
-__device__ __forceinline__ float2 dd_from(double a) {
-  const float h = (float)a;
-  return make_float2(h, (float)(a - (double)h));
-}
+__device__ __forceinline__ float2 dd_from(double a) { return df_split(a); }
 __device__ __forceinline__ float2 dd_norm(float s, float t) {  // fast two-sum, |s| >= |t|
   const float h = s + t;
   return make_float2(h, t - (h - s));

@@ -28,10 +28,28 @@ __global__ void k_split_j(const double2* __restrict__ J, int64_t J_dstride, int6
 }
 
 // ------------------------------------------------------------------ forward traces
-// grid (n_atoms, n_delta * 4), block 256 = 16 x 16 element threads.
-// DF = false: FP64 arithmetic (FP64 form).  DF = true (mixed form): the K x K
-// products and the site sum in double-float arithmetic on the FP32 pipes
+// grid (n_atoms, n_delta * 4), block 256 = 16 x 16 element threads, dynamic smem
+// kubo_smem<DF>().  DF = false: FP64 arithmetic (FP64 form).  DF = true (mixed form): the
+// K x K products and the site sum in double-float arithmetic on the FP32 pipes
 // (unit roundoff about 2^-48; the last trace and everything after it in FP64).
+// Bound by the instruction issues of the double-float products (48 each, about 2.7 k per
+// site and combination and SM).  Two shared-memory stages: the next site's blocks are in
+// flight while this one's are multiplied, two barriers per site; the products of Y are
+// dealt out as (entry, nu) items, so all warps take part.  Measured (2,000 atoms of 59
+// sites, three broadenings): 17.2 ms, of which the integer form of df_split saved 2.1
+// (the FP64 pipe was 59 % busy with it), against 21.5 with one stage, four barriers and
+// an entry's three nu in one thread; the sums keep their order.
+template <bool DF>
+struct KuboShared {
+  using V = typename std::conditional<DF, float4, double2>::type;
+  V T1[2][16][17], T2[2][16][17];
+  V B[2][3][16][17];
+  V P[2][3][16][17];
+  unsigned Jr[2][3][16];  // bit t of Jr[.][nu][x]: J^{n nu}(x, t) != 0
+  double2 red[9][8];
+  int list[256], warp_cnt[8];
+};
+
 template <bool DF>
 __global__ void __launch_bounds__(256) k_kubo_partial(const int64_t* __restrict__ offsets,
                                                       const int32_t* __restrict__ site_atom,
@@ -56,9 +74,8 @@ __global__ void __launch_bounds__(256) k_kubo_partial(const int64_t* __restrict_
     if constexpr (DF) return Jdfd[idx];
     else return Jd[idx];
   };
-  __shared__ V sT1[16][17], sT2[16][17];
-  __shared__ V sB[3][16][17];
-  __shared__ V sP[3][16][17];
+  extern __shared__ __align__(16) unsigned char kubo_raw[];
+  KuboShared<DF>& sh = *reinterpret_cast<KuboShared<DF>*>(kubo_raw);
   auto ld = [](double2 x) -> V {
     if constexpr (DF) return df_split(x);
     else return x;
@@ -87,100 +104,112 @@ __global__ void __launch_bounds__(256) k_kubo_partial(const int64_t* __restrict_
   const int i = tid >> 4, j = tid & 15, lane = tid & 31, warp = tid >> 5;
   const bool act = (i < K) && (j < K);
   const int spm = min(max(0, species[m]), n_species - 1);
-  auto load_jm = [&]() {  // J^{m mu} of the swapped combination, into sB
+  auto load_jm = [&](int buf) {  // J^{m mu} of the swapped combination
     if (act) {
 #pragma unroll
-      for (int u = 0; u < 3; ++u) sB[u][i][j] = ldJ((((size_t)spm * 4 + cb) * 3 + u) * KK + i * K + j);
+      for (int u = 0; u < 3; ++u) sh.B[buf][u][i][j] = ldJ((((size_t)spm * 4 + cb) * 3 + u) * KK + i * K + j);
     }
   };
   // The trace Tr[J^{m mu} Y^nu] reads Y^nu(i, j) only where J^{m mu}(j, i) != 0
   // for some mu (the dipole J: at most 3 of 16 entries per row), so only those
-  // entries of Y are accumulated, each by one thread of a compacted list.
-  __shared__ int sList[256], sWarpCnt[8];
-  __shared__ unsigned sJr[3][16];  // bit t of sJr[nu][x]: J^{n nu}(x, t) != 0
-  load_jm();
+  // entries of Y are accumulated: item x = (nu, entry) of the compacted list.
+  load_jm(0);
   __syncthreads();
-  int cnt = 0, my = -1;
+  int cnt = 0;
   {
-    const bool need = act && (nz(sB[0][j][i]) || nz(sB[1][j][i]) || nz(sB[2][j][i]));
+    const bool need = act && (nz(sh.B[0][0][j][i]) || nz(sh.B[0][1][j][i]) || nz(sh.B[0][2][j][i]));
     const unsigned bal = __ballot_sync(0xffffffffu, need);
-    if (lane == 0) sWarpCnt[warp] = __popc(bal);
+    if (lane == 0) sh.warp_cnt[warp] = __popc(bal);
     __syncthreads();
     int base = 0;
     for (int w = 0; w < 8; ++w) {
-      if (w < warp) base += sWarpCnt[w];
-      cnt += sWarpCnt[w];
+      if (w < warp) base += sh.warp_cnt[w];
+      cnt += sh.warp_cnt[w];
     }
-    if (need) sList[base + __popc(bal & ((1u << lane) - 1u))] = tid;
+    if (need) sh.list[base + __popc(bal & ((1u << lane) - 1u))] = tid;
     __syncthreads();
-    if (tid < cnt) my = sList[tid];
   }
-  const int yi = my >> 4, yj = my & 15;
+  int item[3];  // nu * 256 + entry of this thread's items; -1: none
   Acc Y[3];
 #pragma unroll
-  for (int v = 0; v < 3; ++v) Y[v] = zero();
+  for (int v = 0; v < 3; ++v) {
+    const int x = tid + 256 * v;
+    item[v] = x < 3 * cnt ? x / cnt * 256 + sh.list[x % cnt] : -1;
+    Y[v] = zero();
+  }
   const int64_t s0 = offsets[m], s1 = offsets[m + 1];
-  for (int64_t s = s0; s < s1; ++s) {
+  double2 t1 = mk(0.0, 0.0), t2 = mk(0.0, 0.0);
+  V jv[3] = {V{}, V{}, V{}};
+  auto fetch = [&](int64_t s) {  // site s's blocks into registers
+    if (!act || s >= s1) return;
     const int sp = min(max(0, species[site_atom[s]]), n_species - 1);  // out-of-range ids never index J
-    if (act) {
-      sT1[i][j] = ld(tau[((size_t)e1 * S_total + s) * KK + i * K + j]);
-      sT2[i][j] = ld(tau[((size_t)e2 * S_total + s) * KK + i * K + j]);
+    t1 = tau[((size_t)e1 * S_total + s) * KK + i * K + j];
+    t2 = tau[((size_t)e2 * S_total + s) * KK + i * K + j];
 #pragma unroll
-      for (int v = 0; v < 3; ++v) sB[v][i][j] = ldJ((((size_t)sp * 4 + c) * 3 + v) * KK + i * K + j);
+    for (int v = 0; v < 3; ++v) jv[v] = ldJ((((size_t)sp * 4 + c) * 3 + v) * KK + i * K + j);
+  };
+  fetch(s0);
+  for (int64_t s = s0; s < s1; ++s) {
+    const int buf = (int)((s - s0) & 1);
+    if (act) {
+      sh.T1[buf][i][j] = ld(t1);
+      sh.T2[buf][i][j] = ld(t2);
     }
-    __syncthreads();
 #pragma unroll
     for (int v = 0; v < 3; ++v) {
-      const unsigned br = __ballot_sync(0xffffffffu, act && nz(sB[v][i][j]));
-      if (j == 0) sJr[v][i] = (br >> (lane & 16)) & 0xffffu;
+      if (act) sh.B[buf][v][i][j] = jv[v];
+      const unsigned br = __ballot_sync(0xffffffffu, act && nz(jv[v]));
+      if (j == 0) sh.Jr[buf][v][i] = (br >> (lane & 16)) & 0xffffu;
     }
-    __syncthreads();
+    __syncthreads();  // this stage is complete (and every thread is past the one before it)
+    fetch(s + 1);
     if (act) {
 #pragma unroll
       for (int v = 0; v < 3; ++v) {  // J^nu tau^{n0}(z2) over the nonzero entries of J's row i
         Acc acc = zero();
-        for (unsigned b = sJr[v][i]; b; b &= b - 1) {
+        for (unsigned b = sh.Jr[buf][v][i]; b; b &= b - 1) {
           const int q = __ffs(b) - 1;
-          mac(acc, sB[v][i][q], sT2[q][j]);
+          mac(acc, sh.B[buf][v][i][q], sh.T2[buf][q][j]);
         }
-        sP[v][i][j] = val(acc);
+        sh.P[buf][v][i][j] = val(acc);
       }
     }
     __syncthreads();
-    if (my >= 0) {
 #pragma unroll
-      for (int v = 0; v < 3; ++v)
-        for (int q = 0; q < K; ++q) mac(Y[v], sT1[q][yi], sP[v][q][yj]);  // tau^{0n}(z1) = tau^{n0}(z1)^T
+    for (int v = 0; v < 3; ++v) {
+      if (item[v] < 0) continue;
+      const int nu = item[v] >> 8, yi = (item[v] >> 4) & 15, yj = item[v] & 15;
+#pragma unroll 4
+      for (int q = 0; q < K; ++q)  // tau^{0n}(z1) = tau^{n0}(z1)^T
+        mac(Y[v], sh.T1[buf][q][yi], sh.P[buf][nu][q][yj]);
     }
-    __syncthreads();
   }
+  __syncthreads();
   // S[mu][nu] = Tr[J^{m mu} Y^nu] = sum_ij Jm[i][j] Y[j][i]; entries outside the list are 0
   if (act) {
 #pragma unroll
-    for (int v = 0; v < 3; ++v) sP[v][i][j] = V{};
+    for (int v = 0; v < 3; ++v) sh.P[0][v][i][j] = V{};
   }
-  load_jm();
+  load_jm(0);
   __syncthreads();
-  if (my >= 0) {
 #pragma unroll
-    for (int v = 0; v < 3; ++v) sP[v][yi][yj] = val(Y[v]);
-  }
+  for (int v = 0; v < 3; ++v)
+    if (item[v] >= 0) sh.P[0][item[v] >> 8][(item[v] >> 4) & 15][item[v] & 15] = val(Y[v]);
   __syncthreads();
-  __shared__ double2 red[9][8];
   for (int u = 0; u < 3; ++u)
     for (int v = 0; v < 3; ++v) {
-      double2 t = act ? cmul(wide(sB[u][i][j]), wide(sP[v][j][i])) : mk(0.0, 0.0);
+      double2 t = act ? cmul(wide(sh.B[0][u][i][j]), wide(sh.P[0][v][j][i])) : mk(0.0, 0.0);
 #pragma unroll
       for (int off = 16; off; off >>= 1) {
         t.x += __shfl_xor_sync(0xffffffffu, t.x, off);
         t.y += __shfl_xor_sync(0xffffffffu, t.y, off);
       }
-      if (lane == 0) red[u * 3 + v][warp] = t;
+      if (lane == 0) sh.red[u * 3 + v][warp] = t;
     }
   __syncthreads();
   if (tid < 9) {
     double2 t = mk(0.0, 0.0);
-    for (int w = 0; w < 8; ++w) t = cadd(t, red[tid][w]);
+    for (int w = 0; w < 8; ++w) t = cadd(t, sh.red[tid][w]);
     partial[((size_t)(d * 4 + c) * n_atoms + m) * 9 + tid] = t;
   }
 }
@@ -524,10 +553,24 @@ __global__ void __launch_bounds__(256) k_adj_species(const int32_t* __restrict__
 }
 
 // ------------------------------------------------------------------ wrappers
+static int kubo_partial_attr() {  // more than 48 KB of dynamic shared memory
+  static bool attr_set = false;
+  if (!attr_set) {
+    LSMS_CUDA_TRY(cudaFuncSetAttribute(k_kubo_partial<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)sizeof(KuboShared<true>)));
+    LSMS_CUDA_TRY(cudaFuncSetAttribute(k_kubo_partial<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)sizeof(KuboShared<false>)));
+    attr_set = true;
+  }
+  return LSMS_OK;
+}
+
 int kubo_forward(const int64_t* offsets, const int32_t* site_atom, const int32_t* species, int n_species,
                  const double2* J, int64_t J_dstride, const double2* tau, int64_t S_total, int K, int n_atoms, int n_delta,
                  double volume, bool df, float4* jdf, double2* partial, double2* S, double2* sigma_tilde,
                  double2* sigma, double* rho, cudaStream_t st, int32_t* halve) {
+  const int rc = kubo_partial_attr();
+  if (rc) return rc;
   if (halve) {
     const int n_dj = J_dstride > 0 ? n_delta : 1;
     LSMS_LAUNCH(k_check_conj_j, dim3(1), dim3(256), 0, st, J, J_dstride > 0 ? J_dstride : 0, n_dj,
@@ -537,10 +580,10 @@ int kubo_forward(const int64_t* offsets, const int32_t* site_atom, const int32_t
     const int64_t per = (int64_t)n_species * 12 * K * K;
     const int n_dj = J_dstride > 0 ? n_delta : 1;
     LSMS_LAUNCH(k_split_j, dim3((unsigned)((per + 255) / 256), n_dj), dim3(256), 0, st, J, J_dstride, per, jdf);
-    LSMS_LAUNCH(k_kubo_partial<true>, dim3(n_atoms, n_delta * 4), dim3(256), 0, st, offsets, site_atom, species, J,
+    LSMS_LAUNCH(k_kubo_partial<true>, dim3(n_atoms, n_delta * 4), dim3(256), sizeof(KuboShared<true>), st, offsets, site_atom, species, J,
                 J_dstride, jdf, J_dstride > 0 ? per : 0, tau, S_total, K, n_atoms, n_species, halve, partial);
   } else {
-    LSMS_LAUNCH(k_kubo_partial<false>, dim3(n_atoms, n_delta * 4), dim3(256), 0, st, offsets, site_atom, species, J,
+    LSMS_LAUNCH(k_kubo_partial<false>, dim3(n_atoms, n_delta * 4), dim3(256), sizeof(KuboShared<false>), st, offsets, site_atom, species, J,
                 J_dstride, nullptr, 0, tau, S_total, K, n_atoms, n_species, halve, partial);
   }
   LSMS_LAUNCH(k_kubo_reduce, dim3(n_delta * 4 * 9), dim3(256), 0, st, partial, n_atoms, halve, S);
@@ -559,14 +602,16 @@ __global__ void k_cscale(double2* __restrict__ x, int64_t n, double a) {
 int kubo_atoms(const int64_t* offsets, const int32_t* site_atom, const int32_t* species, int n_species,
                const double2* J, int64_t J_dstride, const double2* tau, int64_t S_total, int K, int n_atoms,
                int n_delta, double volume, bool df, float4* jdf, double2* out, cudaStream_t st) {
+  const int rc = kubo_partial_attr();
+  if (rc) return rc;
   if (df) {
     const int64_t per = (int64_t)n_species * 12 * K * K;
     const int n_dj = J_dstride > 0 ? n_delta : 1;
     LSMS_LAUNCH(k_split_j, dim3((unsigned)((per + 255) / 256), n_dj), dim3(256), 0, st, J, J_dstride, per, jdf);
-    LSMS_LAUNCH(k_kubo_partial<true>, dim3(n_atoms, n_delta * 4), dim3(256), 0, st, offsets, site_atom, species, J,
+    LSMS_LAUNCH(k_kubo_partial<true>, dim3(n_atoms, n_delta * 4), dim3(256), sizeof(KuboShared<true>), st, offsets, site_atom, species, J,
                 J_dstride, jdf, J_dstride > 0 ? per : 0, tau, S_total, K, n_atoms, n_species, nullptr, out);
   } else {
-    LSMS_LAUNCH(k_kubo_partial<false>, dim3(n_atoms, n_delta * 4), dim3(256), 0, st, offsets, site_atom, species, J,
+    LSMS_LAUNCH(k_kubo_partial<false>, dim3(n_atoms, n_delta * 4), dim3(256), sizeof(KuboShared<false>), st, offsets, site_atom, species, J,
                 J_dstride, nullptr, 0, tau, S_total, K, n_atoms, n_species, nullptr, out);
   }
   const int64_t cnt = (int64_t)n_delta * 4 * n_atoms * 9;

@@ -22,10 +22,11 @@
 // y_b = T_b^{-1} x_b with the stored inverse of the diagonal block, then the group's
 // remaining rows.
 //
-// Measured (1,488 units of n about 850, two solves each): 16 columns 7.2 ms, 32
-// columns 9.6 ms, against 11.2 and 18.4 ms (two slices of 16) for chains with the row
+// Measured (1,488 units of n about 850, two solves each): 16 columns 6.4 ms, 32
+// columns 8.9 ms, against 11.2 and 18.4 ms (two slices of 16) for chains with the row
 // updates on the FP32 pipes; the refined tau's error against 64 bits fell (n = 688:
-// 2.35e-11 to 1.74e-11).  Without the L2 requests ahead 8.1 and 11.0 ms.  What is left
+// 2.35e-11 to 1.74e-11).  Without the L2 requests ahead 8.1 and 11.0 ms, and with loads instead of
+// asynchronous copies of the group's blocks 7.2 and 9.6 ms.  What is left
 // above the factor's read (2.5 ms each) is latency: two CTAs per SM, each a chain of
 // split, product and wait per block and of 4 dependent blocks per group.
 #include <cstdint>
