@@ -448,6 +448,165 @@ __global__ void __cluster_dims__(kPanelCluster, 1, 1) __launch_bounds__(kCluster
   cluster.sync();  // no CTA leaves while others may still read its shared memory
 }
 
+// ------------------------------------------------------------------ panels in distributed shared memory
+// The same panel held in the shared memory of a cluster of CL CTAs per unit: CTA r
+// owns the physical rows [r per, (r + 1) per), per = ceil(m / CL), one row per thread;
+// pivots, arithmetic and the logical row numbers as in k_panel_smem.  Per column each
+// CTA reduces its best candidate, forms its reciprocal once (a complex128 division by
+// every warp took a third of a column's FP64 time) and pushes the candidate's row to
+// every CTA of the cluster; after one cluster barrier each CTA has all candidates' rows
+// locally and takes the same pivot (CL = 1: the same without the cluster).  Magnitudes are compared as integers (the bit
+// patterns of non-negative numbers order like their values), not on the FP64 pipe.
+// What bounds it: complex128, the FP64 multiply-adds of the update, shared by CL SMs;
+// complex64, the column's chain of reduction, push and barrier.  For panels that one
+// CTA's shared memory does not hold, and for complex128 where few units would leave SMs
+// idle.  Measured per matrix set: 216 of n = 688 in complex128 17.5 -> 10.5 ms for all
+// panels (the 8 tallest 10.8 -> 5.6, before with rows in L2 on one CTA per unit), 108 of
+// n = 2192 in complex64 22.2 -> 8.4 ms, 20 of n = 160 in complex128 0.79 -> 0.72.
+__device__ __forceinline__ unsigned long long mag_key(float v) {  // NaN, non-candidates (negative): 0
+  return v >= 0.f ? (unsigned long long)__float_as_uint(v) + 1ull : 0ull;
+}
+__device__ __forceinline__ unsigned long long mag_key(double v) {
+  const long long b = __double_as_longlong(v);
+  return b >= 0 && b <= 0x7ff0000000000000ll ? (unsigned long long)b + 1ull : 0ull;
+}
+// warp-wide best (largest key, then lowest logical row) with its tag
+__device__ __forceinline__ void warp_best_key(unsigned long long& key, int& lg, int& tag) {
+  const unsigned hi = (unsigned)(key >> 32), mh = __reduce_max_sync(0xffffffffu, hi);
+  const unsigned lo = hi == mh ? (unsigned)key : 0u, ml = __reduce_max_sync(0xffffffffu, lo);
+  const bool c = hi == mh && lo == ml;
+  const unsigned l = __reduce_min_sync(0xffffffffu, c ? (unsigned)lg : 0xffffffffu);
+  const int src = __ffs(__ballot_sync(0xffffffffu, c && (unsigned)lg == l)) - 1;
+  tag = __shfl_sync(0xffffffffu, tag, src);
+  key = ((unsigned long long)mh << 32) | ml;
+  lg = (int)l;
+}
+
+template <typename R>
+constexpr int kDsmRows = 212992 / (32 * (int)sizeof(Cx<R>));  // rows per CTA: 832 complex64, 416 complex128
+
+template <typename R, int NB, int CL>
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(1024, 1)
+    k_panel_dsm(const Unit* __restrict__ units, char* fac_base, int k, int32_t* stat, int min_rows) {
+  using C = Cx<R>;
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = (int)cluster.block_rank();
+  const Unit u = units[blockIdx.y];
+  const int n = u.n;
+  const int m = n - k;
+  if (m <= 0 || m <= min_rows) return;  // the same for every CTA of the cluster (one unit)
+  const int per = (m + CL - 1) / CL;
+  if (per > (int)blockDim.x || per > kDsmRows<R>) return;  // the launch is sized for the tallest panel
+  extern __shared__ __align__(16) unsigned char panel_raw[];
+  C* sP = reinterpret_cast<C*>(panel_raw);  // [NB][per], column-major, physical rows
+  C* A = reinterpret_cast<C*>(fac_base + u.fac_off);
+  int32_t* piv = reinterpret_cast<int32_t*>(fac_base + u.piv_off);
+  const int nbp = min(NB, m);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  __shared__ unsigned long long c_key[2][CL], w_key[32];
+  __shared__ int c_lg[2][CL], c_ph[2][CL], w_lg[32], w_ph[32];
+  __shared__ C c_rcp[2][CL], c_row[2][CL][NB];
+  const int rbeg = rank * per;
+  const bool own = tid < per && rbeg + tid < m;  // this thread's physical row is rbeg + tid
+  if (own)
+    for (int c = 0; c < nbp; ++c) cp_async_elem(&sP[c * per + tid], &A[(size_t)(k + c) * n + k + rbeg + tid]);
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  int lg = rbeg + tid;
+  auto mag = [](C v) -> R {  // |Re| + |Im|; NaN below every number
+    const R a = cabs1(v);
+    return a >= R(0) ? a : R(-0.5);
+  };
+  // the CTA's candidate for column j to every CTA of the cluster, parity slot par
+  auto publish = [&](unsigned long long key, int l, int j, int par) {
+    int ph = tid;
+    warp_best_key(key, l, ph);
+    if (lane == 0) {
+      w_key[warp] = key;
+      w_lg[warp] = l;
+      w_ph[warp] = ph;
+    }
+    __syncthreads();
+    if (warp == 0) {
+      key = lane < nw ? w_key[lane] : 0ull;
+      l = lane < nw ? w_lg[lane] : m;
+      ph = lane < nw ? w_ph[lane] : 0;
+      warp_best_key(key, l, ph);
+      const C v = (l < m && lane < nbp) ? sP[lane * per + ph] : mk(R(0), R(0));
+      C pv;
+      pv.x = __shfl_sync(0xffffffffu, v.x, j);
+      pv.y = __shfl_sync(0xffffffffu, v.y, j);
+      const C rcp = (pv.x == R(0) && pv.y == R(0)) ? mk(R(0), R(0)) : crcp(pv);
+#pragma unroll
+      for (int r = 0; r < CL; ++r) *cluster.map_shared_rank(&c_row[par][rank][lane], r) = v;
+      if (lane < CL) {
+        *cluster.map_shared_rank(&c_key[par][rank], lane) = key;
+        *cluster.map_shared_rank(&c_lg[par][rank], lane) = l;
+        *cluster.map_shared_rank(&c_ph[par][rank], lane) = rbeg + ph;
+        *cluster.map_shared_rank(&c_rcp[par][rank], lane) = rcp;
+      }
+    }
+    cluster.sync();
+  };
+  cluster.sync();  // every CTA of the cluster has started: its shared memory may be written
+  publish(own ? mag_key(mag(sP[tid])) : 0ull, own ? lg : m, 0, 0);
+  int flags = 0;
+  bool dead = false;  // LSMS_DEBUG_BOUNDS: a pivot index out of range stops the panel (cluster-uniform)
+#pragma unroll 1
+  for (int j = 0; j < nbp && !dead; ++j) {
+    const int par = j & 1;
+    unsigned long long key = lane < CL ? c_key[par][lane] : 0ull;
+    int p = lane < CL ? c_lg[par][lane] : m, w = lane < CL ? lane : 0;
+    warp_best_key(key, p, w);
+    if (kDebugBounds) {
+      int32_t* sw = &stat[u.stat_off];
+      if (!(dbg_in(p, j, m, sw) & dbg_in(c_ph[par][w], 0, m, sw))) {
+        if (rank == 0 && tid == 0)
+          for (int jj = j; jj < nbp; ++jj) piv[k + jj] = k + jj;
+        dead = true;
+        continue;
+      }
+    }
+    if (rank == 0 && tid == 0) piv[k + j] = k + p;
+    lg = lg == j ? p : (lg == p ? j : lg);  // interchange logical rows j and p
+    const C* row = c_row[par][w];
+    const C pv = row[j], rcp = c_rcp[par][w];
+    const bool zero = (pv.x == R(0) && pv.y == R(0));
+    if (zero) flags |= LSMS_UNIT_ZERO_PIVOT;
+    if (!finite2(pv)) flags |= LSMS_UNIT_NONFINITE;
+    unsigned long long bk = 0ull;
+    int bl = m;
+    if (own && lg > j) {
+      const C l = cmul(sP[j * per + tid], rcp);
+      if (!zero) sP[j * per + tid] = l;
+#pragma unroll
+      for (int c = j + 1; c < NB; ++c) {
+        if (c < nbp) {
+          const C v = cfms(l, row[c], sP[c * per + tid]);
+          sP[c * per + tid] = v;
+          if (c == j + 1) {
+            bk = mag_key(mag(v));
+            bl = lg;
+          }
+        }
+      }
+    }
+    if (j + 1 < nbp) publish(bk, bl, j + 1, par ^ 1);
+  }
+  // write back in logical order (every CTA has loaded its rows before the first barrier)
+  if (own && dbg_in(lg, 0, m, &stat[u.stat_off]))
+    for (int c = 0; c < nbp; ++c) A[(size_t)(k + c) * n + k + lg] = sP[c * per + tid];
+  if (rank == 0 && tid == 0 && flags) atomicOr(&stat[u.stat_off], flags);
+  if constexpr (std::is_same<R, float>::value) {
+    float umax = 0.f;
+    if (own && lg < nbp)
+      for (int c = lg; c < nbp; ++c) umax = fmaxf(umax, cabs1(sP[c * per + tid]));
+    const float wm = warp_max_nonneg(umax);
+    if (lane == 0 && wm > 0.f)
+      atomic_max_nonneg(reinterpret_cast<float*>(fac_base + u.m64_off + growth_rel_off(n)) + 1, wm);
+  }
+}
+
 // ------------------------------------------------------------------ swap + trsm
 // Columns right of the panel, one thread per column (256 columns per CTA): the
 // panel's row interchanges, then U12 = L11^{-1} A12.  The 32 interchanges are
@@ -1105,17 +1264,47 @@ __global__ void __launch_bounds__(256) k_step_final(const Unit* __restrict__ uni
 }
 
 // ------------------------------------------------------------------ wrappers
+template <typename R, int CL>
+static int panel_dsm(const Unit* d_units, int n_units, char* fac_base, int k, int32_t* stat, int m_max, int min_rows,
+                     cudaStream_t st) {
+  static bool attr_set = false;
+  if (!attr_set) {
+    LSMS_CUDA_TRY(cudaFuncSetAttribute(k_panel_dsm<R, 32, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       kDsmRows<R> * 32 * (int)sizeof(Cx<R>)));
+    attr_set = true;
+  }
+  const int per = (m_max + CL - 1) / CL;
+  LSMS_LAUNCH((k_panel_dsm<R, 32, CL>), dim3(CL, n_units), dim3((per + 31) / 32 * 32),
+              (size_t)per * 32 * sizeof(Cx<R>), st, d_units, fac_base, k, stat, min_rows);
+  return LSMS_OK;
+}
+
+// CTAs per unit of k_panel_dsm for panels of up to m_max rows; 0: taller than 8 CTAs hold, or
+// complex64 panels that one CTA of k_panel_smem holds (max_rows).
+template <typename R>
+static int panel_cluster_size(int n_units, int m_max, int max_rows) {
+  if (m_max > 8 * kDsmRows<R>) return 0;
+  if (sizeof(R) == 4 && m_max <= max_rows) return 0;
+  int cl = sizeof(R) == 4 ? 2 : 1;
+  while ((m_max + cl - 1) / cl > kDsmRows<R>) cl *= 2;
+  // complex128: also while the clusters leave SMs idle and a CTA keeps 48 rows or more
+  if (sizeof(R) == 8)
+    while (cl < 8 && 2 * cl * n_units <= 152 && m_max >= 96 * cl) cl *= 2;
+  return cl;
+}
+
 template <typename R>
 int lu_factor_chunk(const Unit* d_units, int n_units, int n_max, char* fac_base, int32_t* stat,
                     cudaStream_t st) {
   constexpr int NB = LuCfg<R>::NB;
-  // panels up to kPanelSmemBytes stay in shared memory; taller ones use k_panel
+  // rows of a panel that one CTA holds: k_panel_smem (complex64), k_panel_dsm (complex128)
   constexpr int kPanelSmemBytes = 224 * 1024;
-  const int max_rows = kPanelSmemBytes / (NB * (int)sizeof(Cx<R>));
+  const int max_rows = sizeof(R) == 8 ? kDsmRows<R> : kPanelSmemBytes / (NB * (int)sizeof(Cx<R>));
   static bool attr_set = false;
   if (!attr_set) {
-    LSMS_CUDA_TRY(cudaFuncSetAttribute(k_panel_smem<R, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       kPanelSmemBytes));
+    if constexpr (std::is_same<R, float>::value)
+      LSMS_CUDA_TRY(cudaFuncSetAttribute(k_panel_smem<R, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         kPanelSmemBytes));
     if (sizeof(Cx<R>) == 8)
       LSMS_CUDA_TRY(cudaFuncSetAttribute(k_swap_trsm<R, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          kSwapTileBytes));
@@ -1123,20 +1312,37 @@ int lu_factor_chunk(const Unit* d_units, int n_units, int n_max, char* fac_base,
   }
   for (int k = 0; k < n_max; k += NB) {
     const int m_max = n_max - k;
-    if (m_max > max_rows) {
-      // taller panels on one CTA per unit, or, from 2048 rows (few units of large LIZ
-      // matrices: the single CTA would leave most SMs idle), on a cluster of CTAs per unit
-      if (m_max > 2048 && (m_max + kPanelCluster - 1) / kPanelCluster <= kClusterRows * kClusterThreads)
+    const int cl = panel_cluster_size<R>(n_units, m_max, max_rows);
+    if (cl == 0 && m_max > max_rows) {
+      // taller panels: rows in L2, on a cluster of CTAs per unit as far as its threads reach
+      if ((m_max + kPanelCluster - 1) / kPanelCluster <= kClusterRows * kClusterThreads)
         LSMS_LAUNCH((k_panel_cluster<R, NB>), dim3(kPanelCluster, n_units), dim3(kClusterThreads), 0, st, d_units,
                     fac_base, k, stat, max_rows);
       else
         LSMS_LAUNCH((k_panel<R, NB>), dim3(n_units), dim3(1024), 0, st, d_units, fac_base, k, stat, max_rows);
     }
-    const int rows_smem = std::min(m_max, max_rows);
-    // one thread per row: short panels launch fewer threads, so more CTAs fit on an SM
-    const int threads = std::min(kPanelThreads, (rows_smem + 31) / 32 * 32);
-    LSMS_LAUNCH((k_panel_smem<R, NB>), dim3(n_units), dim3(threads), (size_t)rows_smem * NB * sizeof(Cx<R>), st,
-                d_units, fac_base, k, stat, max_rows);
+    if constexpr (std::is_same<R, double>::value) {
+      // every panel that 8 CTAs hold (beside a taller one: the units whose panel one CTA holds)
+      const int rows = cl ? m_max : max_rows;
+      const int rc = cl <= 1   ? panel_dsm<R, 1>(d_units, n_units, fac_base, k, stat, rows, 0, st)
+                     : cl == 2 ? panel_dsm<R, 2>(d_units, n_units, fac_base, k, stat, rows, 0, st)
+                     : cl == 4 ? panel_dsm<R, 4>(d_units, n_units, fac_base, k, stat, rows, 0, st)
+                               : panel_dsm<R, 8>(d_units, n_units, fac_base, k, stat, rows, 0, st);
+      if (rc) return rc;
+    } else {
+      // units whose panel one CTA holds stay with k_panel_smem
+      if (cl) {
+        const int rc = cl == 2   ? panel_dsm<R, 2>(d_units, n_units, fac_base, k, stat, m_max, max_rows, st)
+                       : cl == 4 ? panel_dsm<R, 4>(d_units, n_units, fac_base, k, stat, m_max, max_rows, st)
+                                 : panel_dsm<R, 8>(d_units, n_units, fac_base, k, stat, m_max, max_rows, st);
+        if (rc) return rc;
+      }
+      const int rows_smem = std::min(m_max, max_rows);
+      // one thread per row: short panels launch fewer threads, so more CTAs fit on an SM
+      const int threads = std::min(kPanelThreads, (rows_smem + 31) / 32 * 32);
+      LSMS_LAUNCH((k_panel_smem<R, NB>), dim3(n_units), dim3(threads), (size_t)rows_smem * NB * sizeof(Cx<R>), st,
+                  d_units, fac_base, k, stat, max_rows);
+    }
     const int trail = n_max - k - NB;
     if (trail <= 0) continue;
     // one warp per column right of the panel
