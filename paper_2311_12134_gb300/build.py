@@ -21,7 +21,7 @@ BUILD_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "liblsmskubo.so")
 LIB_DEBUG = os.path.join(OUT_DIR, "liblsmskubo_debug.so")
 
-CUDA_SOURCES = ["api.cu", "lu.cu", "kubo.cu", "tc_gemm.cu", "tc_gemm64.cu", "tc_solve.cu", "resid_tc.cu"]
+CUDA_SOURCES = ["api.cu", "lu.cu", "kubo.cu", "tc_gemm.cu", "tc_gemm64.cu", "tc_gemm96.cu", "tc_solve.cu", "resid_tc.cu"]
 CXX_SOURCES = ["host.cpp"]
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 

@@ -280,8 +280,13 @@ int solve_tc_chunk(const Unit* d_units, int n_units, const char* fac_base, char*
 int step_tc_chunk(const Unit* d_units, int n_units, int n_max, const char* fac_base, char* ws, int nrhs,
                   const int32_t* done, int32_t* stat, int s, bool forward, cudaStream_t st);
 // Trailing update A22 -= L21 U12 of the complex64 LU on the tensor cores (tc_gemm.cu).
-int gemm_tc_chunk(const Unit* d_units, int n_units, int n_max, int k, char* fac_base, int32_t* stat,
+// c_end: columns below it only (the rest of a column block), 0 = all.
+int gemm_tc_chunk(const Unit* d_units, int n_units, int n_max, int k, int c_end, char* fac_base, int32_t* stat,
                   cudaStream_t st);
+// The same with the kBlkK columns of L from K0 at once (tc_gemm96.cu).
+constexpr int kBlkK = 96;  // columns per block of the large complex64 factorizations
+int gemm_tc96_chunk(const Unit* d_units, int n_units, int n_max, int K0, char* fac_base, int32_t* stat,
+                     cudaStream_t st);
 
 // Trailing update of the complex128 LU on the tensor cores, exact bf16 digit products (tc_gemm64.cu).
 int gemm64_tc_chunk(const Unit* d_units, int n_units, int n_max, int k, char* fac_base, int32_t* stat,

@@ -18,6 +18,7 @@
 // tc_gemm64.cu) and k_solve_c64 (complex64) then run blocked forward/backward
 // substitution.
 #include <algorithm>
+#include <climits>
 #include <type_traits>
 
 #include <cooperative_groups.h>
@@ -665,13 +666,13 @@ constexpr int kSwapTileBytes = 32 * (kSwapCols + 1) * 8;  // complex64 panel-row
 // interchanged rows from the tile, solves in registers and puts them back.
 // Rows below the panel that the interchanges reach are read and written directly.
 template <int NB>
-__device__ __forceinline__ void k_swap_trsm_staged(float2* A, int n, int k, int c0, const float2 (*sL)[NB + 1],
+__device__ __forceinline__ void k_swap_trsm_staged(float2* A, int n, int k, int c0, int cols_end, const float2 (*sL)[NB + 1],
                                                    const int* sTgtRow, const int* sSrcRow, const int* sTgtSrc,
                                                    const int* sNt, float* growth_u) {
   extern __shared__ float2 sTile[];  // [NB][kSwapCols + 1]
   constexpr int LD = kSwapCols + 1;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int ncols = min(kSwapCols, n - c0);
+  const int ncols = min(kSwapCols, cols_end - c0);
   // the tile's 256-byte column segments requested into L2 at once (two lines per thread), so
   // the warps' loads below find them there
   for (int x = tid; x < 2 * ncols; x += blockDim.x)
@@ -717,14 +718,15 @@ __device__ __forceinline__ void k_swap_trsm_staged(float2* A, int n, int k, int 
 }
 
 template <typename R, int NB>
-__global__ void __launch_bounds__(256) k_swap_trsm(const Unit* __restrict__ units, char* fac_base, int k,
+__global__ void __launch_bounds__(256) k_swap_trsm(const Unit* __restrict__ units, char* fac_base, int k, int c_end,
                                                    int32_t* stat) {
   using C = Cx<R>;
   static_assert(NB == 32, "one warp of interchanges");
   const Unit u = units[blockIdx.y];
   const int n = u.n;
+  const int cols_end = min(n, c_end);  // columns below it only (the rest of a column block)
   const int c0 = k + NB + blockIdx.x * kSwapCols;
-  if (c0 >= n) return;  // columns right of the panel exist only when the panel is full
+  if (c0 >= cols_end) return;  // columns right of the panel exist only when the panel is full
   C* A = reinterpret_cast<C*>(fac_base + u.fac_off);
   const int32_t* piv = reinterpret_cast<const int32_t*>(fac_base + u.piv_off);
   if (kDebugBounds) {  // the panel's pivots must lie in [k + j, n)
@@ -744,13 +746,13 @@ __global__ void __launch_bounds__(256) k_swap_trsm(const Unit* __restrict__ unit
   }
   if (tid < 32) compose_panel_swaps(piv, k, NB, tid, sStep, sTgtRow, sSrcRow, sTgtSrc, &sNt);
   if constexpr (sizeof(C) == 8) {
-    k_swap_trsm_staged<NB>(A, n, k, c0, sL, sTgtRow, sSrcRow, sTgtSrc, &sNt,
+    k_swap_trsm_staged<NB>(A, n, k, c0, cols_end, sL, sTgtRow, sSrcRow, sTgtSrc, &sNt,
                            reinterpret_cast<float*>(fac_base + u.m64_off + growth_rel_off(n)) + 1);
     return;
   }
   __syncthreads();
   const int c = c0 + tid;
-  if (c >= n) return;
+  if (c >= cols_end) return;
   C* Ac = A + (size_t)c * n;
   C x[NB];
 #pragma unroll
@@ -778,6 +780,192 @@ __global__ void __launch_bounds__(256) k_swap_trsm(const Unit* __restrict__ unit
   }
 #pragma unroll
   for (int i = 0; i < NB; ++i) Ac[k + i] = x[i];
+}
+
+// ------------------------------------------------------------------ column blocks
+// Large complex64 matrices are factored in blocks of 96 columns: three 32-column panels,
+// each followed by the interchanges, triangular solve and update of the block's own
+// remaining columns; then the columns right of the block take all interchanges, the
+// 96 x 96 unit-lower solve and one update with 96 columns of L (k_gemm_tc96), so
+// the trailing matrix is streamed once per 96 columns.  Within a block L has to be in
+// the row order of the block's last panel: k_swap_left applies each panel's
+// interchanges to the block's columns left of it (k_lapack_rows later applies those of
+// the following blocks).
+
+// One column by one warp: the composed interchanges of a panel (compose_panel_swaps).
+__device__ __forceinline__ void swap_column(float2* col, int k, int lane, const int* src, const int* tgt,
+                                            const int* tgt_src, int nt) {
+  const float2 v = col[src[lane]];
+  const float2 t = lane < nt ? col[tgt_src[lane]] : make_float2(0.f, 0.f);
+  __syncwarp();
+  col[k + lane] = v;
+  if (lane < nt) col[tgt[lane]] = t;
+  __syncwarp();
+}
+
+// The interchanges of the panel at k applied to columns [c0, k).  grid (n_units), block 256.
+__global__ void __launch_bounds__(256) k_swap_left(const Unit* __restrict__ units, char* fac_base, int k, int c0,
+                                                   int32_t* stat) {
+  constexpr int NB = 32;
+  const Unit u = units[blockIdx.x];
+  const int n = u.n;
+  if (k >= n) return;
+  float2* A = reinterpret_cast<float2*>(fac_base + u.fac_off);
+  const int32_t* piv = reinterpret_cast<const int32_t*>(fac_base + u.piv_off);
+  const int nbp = min(NB, n - k);
+  if (kDebugBounds) {
+    const bool bad = (int)threadIdx.x < nbp && !dbg_in(piv[k + threadIdx.x], k + threadIdx.x, n, &stat[u.stat_off]);
+    if (__syncthreads_or(bad)) return;
+  }
+  __shared__ int sStep[NB], sTgt[NB], sSrc[NB], sTgtSrc[NB], sNt;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (warp == 0) compose_panel_swaps(piv, k, nbp, lane, sStep, sTgt, sSrc, sTgtSrc, &sNt);
+  __syncthreads();
+  for (int c = c0 + warp; c < k; c += 8) {
+    float2* col = A + (size_t)c * n;
+    if (nbp == NB) {
+      swap_column(col, k, lane, sSrc, sTgt, sTgtSrc, sNt);
+    } else {  // the last, partial panel: rows below it do not exist
+      const float2 v = lane < nbp ? col[sSrc[lane]] : make_float2(0.f, 0.f);
+      __syncwarp();
+      if (lane < nbp) col[k + lane] = v;
+    }
+  }
+}
+
+constexpr int kBlkCols = 64;  // columns per CTA of k_swap_trsm_blk
+constexpr int kBlkPanels = kBlkK / 32;
+constexpr int kBlkSmem = kBlkK * (kBlkCols + 1) * 8 + kBlkK * 32 * 8;
+
+// Columns right of a 96-column block at K0: the interchanges of its three panels, then
+// U12 = L11^{-1} A12 with the 96 x 96 unit-lower L11.  The panels' composed interchanges
+// are composed again into one gather (a row takes the value of the row that the panels,
+// undone from the last to the first, lead to; rows below the block always take a block
+// row's value, because a panel's rows are final after it), so a column costs one round
+// of loads instead of three of loads and stores.  The solve runs 8 rows at a time: one
+// thread per column substitutes, then all threads update the block's remaining rows.
+// grid (ceil(columns / 64), n_units), block 256, dynamic smem kBlkSmem.
+__global__ void __launch_bounds__(256) k_swap_trsm_blk(const Unit* __restrict__ units, char* fac_base, int K0,
+                                                      int32_t* stat) {
+  constexpr int NB = 32, KB = kBlkK, LD = kBlkCols + 1, NPAN = kBlkPanels;
+  const Unit u = units[blockIdx.y];
+  const int n = u.n;
+  const int c0 = K0 + KB + blockIdx.x * kBlkCols;
+  if (c0 >= n) return;  // columns right of the block exist only when the block is full
+  const int ncols = min(kBlkCols, n - c0);
+  float2* A = reinterpret_cast<float2*>(fac_base + u.fac_off);
+  const int32_t* piv = reinterpret_cast<const int32_t*>(fac_base + u.piv_off);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (kDebugBounds) {
+    const bool bad = tid < KB && !dbg_in(piv[K0 + tid], K0 + tid, n, &stat[u.stat_off]);
+    if (__syncthreads_or(bad)) return;
+  }
+  extern __shared__ __align__(16) unsigned char blk_raw[];
+  float2* sT = reinterpret_cast<float2*>(blk_raw);  // [KB][LD] the block's rows of the columns
+  float2* sL = sT + KB * LD;                         // [NB][KB] 32 columns of L11, column-major
+  __shared__ int sStep[NPAN][NB], sTgt[NPAN][NB], sSrc[NPAN][NB], sTgtSrc[NPAN][NB], sNt[NPAN];
+  __shared__ int sFrom[KB];                // block row i takes the value of row sFrom[i]
+  __shared__ int sOut[KB], sOutFrom[KB];   // row sOut[q] below the block takes that of block row sOutFrom[q]
+  __shared__ int sNOut;
+  if (warp < NPAN)
+    compose_panel_swaps(piv, K0 + NB * warp, NB, lane, sStep[warp], sTgt[warp], sSrc[warp], sTgtSrc[warp], &sNt[warp]);
+  if (tid == 0) sNOut = 0;
+  __syncthreads();
+  // the row whose value row r holds after panels 0 .. p
+  auto origin = [&](int r, int p) {
+    for (; p >= 0; --p) {
+      const int k = K0 + NB * p;
+      if (r >= k && r < k + NB) {
+        r = sSrc[p][r - k];
+      } else {
+        for (int q = 0; q < sNt[p]; ++q)
+          if (sTgt[p][q] == r) {
+            r = sTgtSrc[p][q];
+            break;
+          }
+      }
+    }
+    return r;
+  };
+  if (tid < KB) {
+    sFrom[tid] = origin(K0 + tid, NPAN - 1);
+  } else if (tid < 2 * KB) {
+    const int p = (tid - KB) / NB, q = (tid - KB) % NB;
+    if (q < sNt[p] && sTgt[p][q] >= K0 + KB) {
+      const int r = sTgt[p][q];
+      bool later = false;  // a row that a later panel reaches too is listed there
+      for (int pp = p + 1; pp < NPAN; ++pp)
+        for (int qq = 0; qq < sNt[pp]; ++qq) later |= sTgt[pp][qq] == r;
+      if (!later) {
+        const int o = atomicAdd(&sNOut, 1);
+        sOut[o] = r;
+        sOutFrom[o] = origin(r, p);
+      }
+    }
+  }
+  __syncthreads();
+  const int n_out = sNOut;
+  for (int c = warp; c < ncols; c += 8) {
+    float2* col = A + (size_t)(c0 + c) * n;
+    float2 v[NPAN], t[NPAN];
+#pragma unroll
+    for (int p = 0; p < NPAN; ++p) {
+      v[p] = col[sFrom[NB * p + lane]];
+      if (NB * p + lane < n_out) t[p] = col[sOutFrom[NB * p + lane]];
+    }
+    __syncwarp();
+#pragma unroll
+    for (int p = 0; p < NPAN; ++p) {
+      sT[(NB * p + lane) * LD + c] = v[p];
+      if (NB * p + lane < n_out) col[sOut[NB * p + lane]] = t[p];
+    }
+  }
+  float umax = 0.f;  // pivot growth: largest |U12| entry
+  const int c = tid & (kBlkCols - 1), rg = tid >> 6;  // column, row group of 4
+#pragma unroll 1
+  for (int p = 0; p < NPAN; ++p) {
+    __syncthreads();
+    for (int idx = tid; idx < NB * KB; idx += 256) {  // rows NB p .. of columns NB p .. + 31
+      const int r = idx % KB, j = idx / KB;
+      if (r >= NB * p) sL[idx] = A[(size_t)(K0 + NB * p + j) * n + K0 + r];
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int b = 0; b < NB; b += 8) {
+      const int i0 = NB * p + b;
+      if (rg == 0) {
+        float2 x[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[i] = sT[(i0 + i) * LD + c];
+#pragma unroll
+        for (int i = 1; i < 8; ++i)
+#pragma unroll
+          for (int j = 0; j < i; ++j) x[i] = cfms(sL[(b + j) * KB + i0 + i], x[j], x[i]);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          sT[(i0 + i) * LD + c] = x[i];
+          if (c < ncols) umax = fmaxf(umax, cabs1(x[i]));
+        }
+      }
+      __syncthreads();
+      float2 x[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) x[j] = sT[(i0 + j) * LD + c];
+      for (int r = i0 + 8 + rg; r < KB; r += 4) {
+        float2 a = sT[r * LD + c];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) a = cfms(sL[(b + j) * KB + r], x[j], a);
+        sT[r * LD + c] = a;
+      }
+      __syncthreads();
+    }
+  }
+  for (int cc = warp; cc < ncols; cc += 8)
+#pragma unroll
+    for (int p = 0; p < NPAN; ++p) A[(size_t)(c0 + cc) * n + K0 + NB * p + lane] = sT[(NB * p + lane) * LD + cc];
+  const float wm = warp_max_nonneg(umax);
+  if (lane == 0 && wm > 0.f)
+    atomic_max_nonneg(reinterpret_cast<float*>(fac_base + u.m64_off + growth_rel_off(n)) + 1, wm);
 }
 
 // ------------------------------------------------------------------ complex64 solve
@@ -906,8 +1094,10 @@ constexpr int kLapBlocks = 8;  // 32-column blocks of L per CTA of k_lapack_rows
 // g kLapBlocks .. g kLapBlocks + kLapBlocks - 1, after building the composition of
 // the later panels' interchanges itself (the prepends are cheap; the row moves of
 // the blocks run in parallel over the CTAs).
+// grp: panels per column block of the factorization (3: within a block L is in the row order of
+// its last panel already, so block b takes the interchanges of the panels after its column block).
 __global__ void __launch_bounds__(256) k_lapack_rows(const Unit* __restrict__ units, const char* fac_base_c,
-                                                     int n_max, int32_t* stat) {
+                                                     int n_max, int grp, int32_t* stat) {
   constexpr int NB = 32;
   char* fac_base = const_cast<char*>(fac_base_c);
   const Unit u = units[blockIdx.y];
@@ -928,9 +1118,9 @@ __global__ void __launch_bounds__(256) k_lapack_rows(const Unit* __restrict__ un
   for (int r = tid; r < n; r += blockDim.x) idx[r] = pos[r] = (unsigned short)r;
   __syncthreads();
   for (int b = nb - 2; b >= b_lo; --b) {
-    // prepend panel b + 1's interchanges, its last one first
+    // prepend the interchanges of the panel (of the grp panels) that starts after block b, the last first
     if (tid == 0) {
-      const int r0 = NB * (b + 1), r1 = min(n, r0 + NB);
+      const int r0 = NB * (b + 1), r1 = (b + 1) % grp == 0 ? min(n, r0 + NB * grp) : r0;
       for (int r = r1 - 1; r >= r0; --r) {
         const int a = r, c = piv[r];
         if (a != c && dbg_in(c, r, n, &stat[u.stat_off])) {
@@ -1264,6 +1454,9 @@ __global__ void __launch_bounds__(256) k_step_final(const Unit* __restrict__ uni
 }
 
 // ------------------------------------------------------------------ wrappers
+// complex64 matrices from this order on are factored in column blocks.  TWO_LEVEL_MEASURED
+constexpr int kTwoLevelRows = 1200;
+
 template <typename R, int CL>
 static int panel_dsm(const Unit* d_units, int n_units, char* fac_base, int k, int32_t* stat, int m_max, int min_rows,
                      cudaStream_t st) {
@@ -1305,11 +1498,14 @@ int lu_factor_chunk(const Unit* d_units, int n_units, int n_max, char* fac_base,
     if constexpr (std::is_same<R, float>::value)
       LSMS_CUDA_TRY(cudaFuncSetAttribute(k_panel_smem<R, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          kPanelSmemBytes));
-    if (sizeof(Cx<R>) == 8)
+    if (sizeof(Cx<R>) == 8) {
       LSMS_CUDA_TRY(cudaFuncSetAttribute(k_swap_trsm<R, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          kSwapTileBytes));
+      LSMS_CUDA_TRY(cudaFuncSetAttribute(k_swap_trsm_blk, cudaFuncAttributeMaxDynamicSharedMemorySize, kBlkSmem));
+    }
     attr_set = true;
   }
+  const bool two_level = sizeof(R) == 4 && n_max >= kTwoLevelRows;
   for (int k = 0; k < n_max; k += NB) {
     const int m_max = n_max - k;
     const int cl = panel_cluster_size<R>(n_units, m_max, max_rows);
@@ -1343,15 +1539,35 @@ int lu_factor_chunk(const Unit* d_units, int n_units, int n_max, char* fac_base,
       LSMS_LAUNCH((k_panel_smem<R, NB>), dim3(n_units), dim3(threads), (size_t)rows_smem * NB * sizeof(Cx<R>), st,
                   d_units, fac_base, k, stat, max_rows);
     }
+    if constexpr (std::is_same<R, float>::value) {
+      if (two_level) {
+        const int K0 = k / kBlkK * kBlkK, K1 = K0 + kBlkK;
+        if (k > K0) LSMS_LAUNCH(k_swap_left, dim3(n_units), dim3(256), 0, st, d_units, fac_base, k, K0, stat);
+        const int rest = std::min(K1, n_max) - k - NB;  // columns of the block right of the panel
+        if (rest > 0) {
+          LSMS_LAUNCH((k_swap_trsm<R, NB>), dim3(1, n_units), dim3(256), kSwapTileBytes, st, d_units, fac_base, k, K1,
+                      stat);
+          const int rc = gemm_tc_chunk(d_units, n_units, n_max, k, K1, fac_base, stat, st);
+          if (rc) return rc;
+        }
+        if (k + NB == K1 && K1 < n_max) {
+          LSMS_LAUNCH(k_swap_trsm_blk, dim3((n_max - K1 + kBlkCols - 1) / kBlkCols, n_units), dim3(256), kBlkSmem, st,
+                      d_units, fac_base, K0, stat);
+          const int rc = gemm_tc96_chunk(d_units, n_units, n_max, K0, fac_base, stat, st);
+          if (rc) return rc;
+        }
+        continue;
+      }
+    }
     const int trail = n_max - k - NB;
     if (trail <= 0) continue;
-    // one warp per column right of the panel
+    // one thread per column right of the panel
     LSMS_LAUNCH((k_swap_trsm<R, NB>), dim3((trail + kSwapCols - 1) / kSwapCols, n_units), dim3(256),
                 sizeof(Cx<R>) == 8 ? kSwapTileBytes : 0, st, d_units,
-                fac_base, k, stat);
+                fac_base, k, INT_MAX, stat);
     if constexpr (std::is_same<R, float>::value) {
       // complex64: the trailing update runs on the tensor cores (3xTF32, tc_gemm.cu)
-      const int rc = gemm_tc_chunk(d_units, n_units, n_max, k, fac_base, stat, st);
+      const int rc = gemm_tc_chunk(d_units, n_units, n_max, k, 0, fac_base, stat, st);
       if (rc) return rc;
     } else {
       // complex128: exact digit products on the tensor cores (tc_gemm64.cu)
@@ -1374,7 +1590,7 @@ int lu_factor_chunk(const Unit* d_units, int n_units, int n_max, char* fac_base,
     const int nb_max = (n_max + 31) / 32;
     if (nb_max > 1)
       LSMS_LAUNCH(k_lapack_rows, dim3((nb_max - 1 + kLapBlocks - 1) / kLapBlocks, n_units), dim3(256), lap, st,
-                  d_units, fac_base, n_max, stat);
+                  d_units, fac_base, n_max, two_level ? kBlkPanels : 1, stat);
     LSMS_LAUNCH(k_lapack_perm, dim3(n_units), dim3(256), (size_t)n_max * 2, st, d_units, fac_base, stat);
   }
   return LSMS_OK;

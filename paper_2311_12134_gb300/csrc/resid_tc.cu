@@ -357,9 +357,9 @@ __global__ void __launch_bounds__(256, 2) k_residual_tc(const Unit* __restrict__
       // every class) starts from zero.
       const bool fresh = (ch % FLUSH) == 0;
 #pragma unroll
-      for (int ks = 0; ks < 2; ++ks)
+      for (int s = 0; s < ND; ++s)
 #pragma unroll
-        for (int s = 0; s < ND; ++s)
+        for (int ks = 0; ks < 2; ++ks)
           mma_bf16(tmem + (uint32_t)(s * NOUT), make_desc(a0 + s * PLANE_A + ks * 2 * LBO), make_desc(b0 + ks * 2 * LBO),
                    make_idesc(TM, NOUT * (ND - s)), (fresh && ks == 0 && s == 0) ? 0u : 1u);
       asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(

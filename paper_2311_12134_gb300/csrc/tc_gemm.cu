@@ -19,6 +19,7 @@
 //   all threads  wait (bounded), read the accumulator with tcgen05.ld
 //                (warp w owns TMEM lanes 32w..32w+31) and update C in place,
 //                one tile behind the products.
+#include <climits>
 #include <cstdint>
 
 #include "common.cuh"
@@ -128,7 +129,7 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
 // LSMS_UNIT_TIMEOUT, the walk stops, and the CTA waits (bounded) for its last
 // issued product before freeing the accumulators.
 __global__ void __launch_bounds__(128) k_gemm_tc(const Unit* __restrict__ units, char* fac_base, int k,
-                                                 int32_t* stat) {
+                                                 int c_end, int32_t* stat) {
   using namespace tc;
   const Unit u = units[blockIdx.y];
   const int n = u.n;
@@ -137,7 +138,9 @@ __global__ void __launch_bounds__(128) k_gemm_tc(const Unit* __restrict__ units,
   if (mt <= 0) return;
   const int ti = blockIdx.x;
   if (ti * TM >= mt) return;
-  const int tn = (mt + TNC - 1) / TNC;
+  // columns t0 .. min(n, c_end) - 1; loads and stores beyond n are masked, and c_end - t0 is a multiple of 32
+  const int tn = (min(n, c_end) - t0 + TNC - 1) / TNC;
+  if (tn <= 0) return;
   const int row0 = t0 + ti * TM;
   float2* A = reinterpret_cast<float2*>(fac_base + u.fac_off);
 
@@ -331,7 +334,7 @@ __global__ void __launch_bounds__(128) k_gemm_tc(const Unit* __restrict__ units,
   }
 }
 
-int gemm_tc_chunk(const Unit* d_units, int n_units, int n_max, int k, char* fac_base, int32_t* stat,
+int gemm_tc_chunk(const Unit* d_units, int n_units, int n_max, int k, int c_end, char* fac_base, int32_t* stat,
                   cudaStream_t st) {
   static bool attr_set = false;
   if (!attr_set) {
@@ -341,7 +344,8 @@ int gemm_tc_chunk(const Unit* d_units, int n_units, int n_max, int k, char* fac_
   const int mt = n_max - k - tc::NB;
   if (mt <= 0) return LSMS_OK;
   const int tm = (mt + tc::TM - 1) / tc::TM;
-  LSMS_LAUNCH(k_gemm_tc, dim3(tm, n_units), dim3(128), tc::SMEM_BYTES, st, d_units, fac_base, k, stat);
+  LSMS_LAUNCH(k_gemm_tc, dim3(tm, n_units), dim3(128), tc::SMEM_BYTES, st, d_units, fac_base, k,
+              c_end ? c_end : INT_MAX, stat);
   return LSMS_OK;
 }
 

@@ -31,10 +31,13 @@
 #include <cstdint>
 
 #include "common.cuh"
+#include "tc_bf16.cuh"
 
 namespace lsms {
 
 namespace oz {
+
+using namespace tb;  // descriptors, instructions, barriers
 
 constexpr int NB = 32;                // complex panel width
 constexpr int TM = 128;               // rows per CTA (TMEM lanes)
@@ -49,49 +52,7 @@ template <int ND>
 constexpr int kGemmSmem = ND * PLANE_A + 2 * ND * PLANE_B + 4 * TM * 4 + 4 * NCC * 4 + 64 + 1024;
 constexpr uint32_t ACC_COLS = 256;    // columns between the two accumulators (ND * NR used)
 constexpr uint32_t TMEM_COLS = 512;
-constexpr long long kWaitLimit = 1ll << 24;  // bounded mbarrier wait (polls)
 static_assert(NT == TM * 4 && NT == NCC * NB, "tile shape");
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-// K-major operand, 128-byte swizzle, one 128-byte row per matrix row: 8-row groups 1024 B apart.
-__device__ __forceinline__ uint64_t make_desc(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFF) >> 4);
-  d |= (uint64_t)1 << 16;
-  d |= (uint64_t)(1024 >> 4) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)2 << 61;
-  return d;
-}
-
-// kind::f16 with bf16 A and B: D f32, both K-major, N and M.
-__host__ __device__ constexpr uint32_t make_idesc(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      :
-      : "r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(acc));
-}
-
-__device__ __forceinline__ bool mbar_try_wait(uint32_t mbar, uint32_t phase) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(mbar), "r"(phase)
-      : "memory");
-  return ok != 0;
-}
 
 __device__ __forceinline__ void tmem_ld4(uint32_t taddr, float* v) {  // completed by tcgen05.wait::ld
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
@@ -116,9 +77,9 @@ __host__ __device__ constexpr int top_bits() {
 template <int ND>
 __device__ __forceinline__ void issue_tile(uint32_t d, uint32_t a0, uint32_t b0, uint32_t mbar) {
 #pragma unroll
-  for (int ks = 0; ks < 4; ++ks)
+  for (int s = 0; s < ND; ++s)
 #pragma unroll
-    for (int s = 0; s < ND; ++s)
+    for (int ks = 0; ks < 4; ++ks)
       mma_bf16(d + (uint32_t)(s * NR), make_desc(a0 + s * PLANE_A + ks * 32), make_desc(b0 + ks * 32),
                make_idesc(TM, NR * (ND - s)), (ks | s) ? 1u : 0u);
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar) : "memory");
@@ -336,15 +297,7 @@ __global__ void __launch_bounds__(oz::NT, 1) k_gemm64_tc(const Unit* __restrict_
       launch_tile(j + 1);
       issued = it + 1;
     }
-    if (warp == 0) {
-      ok = false;
-      const uint32_t mb = smem_u32(mbar + (it & 1));
-      for (long long q = 0; q < kWaitLimit; ++q)
-        if (mbar_try_wait(mb, (uint32_t)((it >> 1) & 1))) {
-          ok = true;
-          break;
-        }
-    }
+    if (warp == 0) ok = mbar_wait(mbar + (it & 1), (uint32_t)((it >> 1) & 1));
     ok = __syncthreads_and(ok);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (!ok) break;
@@ -372,9 +325,7 @@ __global__ void __launch_bounds__(oz::NT, 1) k_gemm64_tc(const Unit* __restrict_
   if (!ok && tid == 0) {
     atomicOr(&stat[u.stat_off], LSMS_UNIT_TIMEOUT);
     // give the tensor core a second bounded window before the accumulators are freed
-    const uint32_t mb = smem_u32(mbar + (issued & 1));
-    for (long long q = 0; q < kWaitLimit; ++q)
-      if (mbar_try_wait(mb, (uint32_t)((issued >> 1) & 1))) break;
+    mbar_wait(mbar + (issued & 1), (uint32_t)((issued >> 1) & 1));
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -547,14 +498,7 @@ __global__ void __launch_bounds__(oz::NT, 1) k_solve64_tc(const Unit* __restrict
   // products `issued - 1` complete (bounded); CTA-uniform, also the barrier of what came before
   auto wait_products = [&]() -> bool {
     bool w = true;
-    if (warp == 0 && issued > 0) {
-      w = false;
-      for (long long q = 0; q < kWaitLimit; ++q)
-        if (mbar_try_wait(smem_u32(mbar), (uint32_t)((issued - 1) & 1))) {
-          w = true;
-          break;
-        }
-    }
+    if (warp == 0 && issued > 0) w = mbar_wait(mbar, (uint32_t)((issued - 1) & 1));
     w = __syncthreads_and(w);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     return w;
@@ -717,8 +661,7 @@ __global__ void __launch_bounds__(oz::NT, 1) k_solve64_tc(const Unit* __restrict
   }
   if (!ok && tid == 0) {
     atomicOr(&stat[u.stat_off], LSMS_UNIT_TIMEOUT);
-    for (long long q = 0; q < kWaitLimit; ++q)
-      if (mbar_try_wait(smem_u32(mbar), (uint32_t)((issued - 1) & 1))) break;
+    if (issued > 0) mbar_wait(mbar, (uint32_t)((issued - 1) & 1));
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();

@@ -31,22 +31,21 @@
 // split, product and wait per block and of 4 dependent blocks per group.
 #include <cstdint>
 
-#include <cuda_bf16.h>
-
 #include "common.cuh"
+#include "tc_bf16.cuh"
 
 namespace lsms {
 
 namespace ts {
 
+using namespace tb;
+
 constexpr int NB = 32;              // complex K per step, rows per diagonal block
 constexpr int TM = 128;             // rows per group (TMEM lanes)
-constexpr int NP = 3;               // bf16 parts per value, classes per accumulator
 constexpr int NT = 256;
 constexpr int kAhead = 3;           // blocks requested into L2 ahead of their loads
 constexpr int WINDOW = 4;           // steps (128 complex K) between additions into registers
 constexpr int PLANE_A = TM * 128;   // 64 real K x 2 bytes per row, 128-byte swizzle
-constexpr long long kWaitLimit = 1ll << 24;
 
 template <int NCOL> constexpr int kPlaneB = 2 * NCOL * 128;
 template <int NCOL> constexpr int kLdX = NCOL + 2;  // row stride of the group's X in shared memory
@@ -55,70 +54,6 @@ template <int NCOL>
 constexpr int kSmem = NP * PLANE_A + kBBytes<NCOL> + TM * kLdX<NCOL> * 8 + 64 + 1024;
 template <int NCOL> constexpr uint32_t kTmemCols = NP * 2 * NCOL <= 128 ? 128 : 256;
 static_assert((96 + 64 + 32) * NB * 8 == NP * PLANE_A, "a group's off-diagonal blocks fill the A planes");
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-// K-major, 128-byte swizzle, 8-row groups 1024 B apart.
-__device__ __forceinline__ uint64_t make_desc(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFF) >> 4);
-  d |= (uint64_t)1 << 16;
-  d |= (uint64_t)(1024 >> 4) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)2 << 61;
-  return d;
-}
-
-// kind::f16 with bf16 A and B: D f32, both K-major, N and M.
-__host__ __device__ constexpr uint32_t make_idesc(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      :
-      : "r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(acc));
-}
-
-__device__ __forceinline__ bool mbar_try_wait(uint32_t mbar, uint32_t phase) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(mbar), "r"(phase)
-      : "memory");
-  return ok != 0;
-}
-
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {  // completed by tcgen05.wait::ld
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
-               : "r"(taddr));
-}
-
-__device__ __forceinline__ uint32_t bf16_pair(float lo, float hi) {
-  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<const uint32_t*>(&v);
-}
-
-// The three bf16 parts of two values as packed pairs; the remainders are exact in FP32.
-__device__ __forceinline__ void split3(float x0, float x1, uint32_t (&p)[NP]) {
-#pragma unroll
-  for (int s = 0; s < NP; ++s) {
-    p[s] = bf16_pair(x0, x1);
-    if (s + 1 < NP) {
-      x0 -= __uint_as_float(p[s] << 16);
-      x1 -= __uint_as_float(p[s] & 0xffff0000u);
-    }
-  }
-}
 
 }  // namespace ts
 
@@ -167,14 +102,7 @@ __global__ void __launch_bounds__(ts::NT, 2) k_solve_tc(const Unit* __restrict__
   bool ok = true;
   auto wait_products = [&]() -> bool {  // bounded, CTA-uniform
     bool w = true;
-    if (warp == 0 && issued > 0) {
-      w = false;
-      for (long long q = 0; q < kWaitLimit; ++q)
-        if (mbar_try_wait(smem_u32(mbar), (uint32_t)((issued - 1) & 1))) {
-          w = true;
-          break;
-        }
-    }
+    if (warp == 0 && issued > 0) w = mbar_wait(mbar, (uint32_t)((issued - 1) & 1));
     w = __syncthreads_and(w);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     return w;
@@ -308,9 +236,9 @@ __global__ void __launch_bounds__(ts::NT, 2) k_solve_tc(const Unit* __restrict__
       if (tid == 0) {
         const uint32_t a0 = smem_u32(sA), b0 = smem_u32(sB);
 #pragma unroll
-        for (int ks = 0; ks < 4; ++ks)
+        for (int s = 0; s < NP; ++s)
 #pragma unroll
-          for (int s = 0; s < NP; ++s)
+          for (int ks = 0; ks < 4; ++ks)
             mma_bf16(tmem + (uint32_t)(s * 2 * NCOL), make_desc(a0 + s * PLANE_A + ks * 32), make_desc(b0 + ks * 32),
                      make_idesc(TM, 2 * NCOL * (NP - s)), (w | ks | s) ? 1u : 0u);
         asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
@@ -452,8 +380,7 @@ __global__ void __launch_bounds__(ts::NT, 2) k_solve_tc(const Unit* __restrict__
   }
   if (!ok && tid == 0) {
     atomicOr(&stat[u.stat_off], LSMS_UNIT_TIMEOUT);
-    for (long long q = 0; q < kWaitLimit; ++q)
-      if (mbar_try_wait(smem_u32(mbar), (uint32_t)((issued - 1) & 1))) break;
+    mbar_wait(mbar, (uint32_t)((issued - 1) & 1));
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
