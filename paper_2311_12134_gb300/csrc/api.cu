@@ -4,11 +4,11 @@
 // Path per call of lsms_tau_blocks (Eq. tau-inverse on every LIZ):
 //   k_assemble   M = T^{-1} - g, g from Gaunt x h_l(kappa R) x Y_L(R^)
 //   lu (lu.cu)   P M = L U, blocked, all units of a chunk per launch
-//   k_solve      X = M^{-1} E0 -> tau^{p0}
-//   mixed form:  complex64 LU/solves, then k_residual (B - M X to about
-//                2^-48, double-float arithmetic on the FP32 pipes) / k_solve
-//                (complex64 correction) / k_ir_update until the correction is
-//                below 1e-10 of X (at most kIrMaxIter sweeps)
+//   solves       X = M^{-1} E0 -> tau^{p0}
+//   mixed form:  complex64 LU/solves, then the residual B - M X to about 2^-48
+//                (k_residual_tc, or k_residual below 9 columns) / complex64
+//                correction / k_ir_update until the correction is below 1e-10
+//                of X (at most kIrMaxIter sweeps)
 //   k_write_tau  scatter X into tau[e][site]
 #include <algorithm>
 #include <cstdlib>

@@ -5,14 +5,17 @@
 // LIZ matrix M (n = K S, column-major, ld = n) is factored P M = L U in place.
 // Pivoting: the row with the largest |Re| + |Im| in the column, the lowest row
 // on ties.  Right-looking, panel width NB:
-//   k_panel      factor the n-k x NB panel (pivot search by warp shuffles),
+//   the panel    n-k rows x NB columns, pivot search by warp reductions: k_panel_smem
+//                (complex64, one CTA), k_panel_dsm (1 to 8 CTAs' shared memory),
+//                k_panel_cluster / k_panel (taller, rows in L2),
 //   k_swap_trsm  apply the panel's row swaps to the columns right of it and
 //                form U12 = L11^{-1} A12 (one warp per column); columns left
 //                of the panel are not swapped (L is kept as computed, LINPACK
 //                style),
 //   A22 -= L21 U12 on the tensor cores: k_gemm64_tc (tc_gemm64.cu, exact digit
 //                products) for complex128, k_gemm_tc (tc_gemm.cu, 3xTF32) for
-//                complex64.
+//                complex64; from n = 800 in blocks of three panels
+//                (k_swap_trsm_blk, k_gemm_tc96).
 // Units of a chunk are sorted by n (largest first); each launch covers every
 // unit and units already finished return at once.  k_solve64_tc (FP64,
 // tc_gemm64.cu) and k_solve_c64 (complex64) then run blocked forward/backward
@@ -1454,8 +1457,12 @@ __global__ void __launch_bounds__(256) k_step_final(const Unit* __restrict__ uni
 }
 
 // ------------------------------------------------------------------ wrappers
-// complex64 matrices from this order on are factored in column blocks.  TWO_LEVEL_MEASURED
-constexpr int kTwoLevelRows = 1200;
+// complex64 matrices from this order on are factored in column blocks.  Whole calls, 32-column
+// updates / blocks: n = 688 (512 units) 27.1 / 27.0 ms, n = 880 (108) 17.0 / 16.3, n about 850
+// (1,488) 109.2 / 106.3, n = 2192 (108) 62.1 / 53.0, n = 15,440 (4) 880 / 561 ms; tau's error
+// falls with the blocks (n about 850: 2.3e-11 to 1.2e-11).  Below, the gain of the update goes
+// into the 96-wide triangular solve (three times the work of the 32-wide one).
+constexpr int kTwoLevelRows = 800;
 
 template <typename R, int CL>
 static int panel_dsm(const Unit* d_units, int n_units, char* fac_base, int k, int32_t* stat, int m_max, int min_rows,
