@@ -402,8 +402,27 @@ def sparse_product_cmacs(J, species, offsets, site_atom, weights, K):
     return adj, trace
 
 
+BLOCK_N, BLOCK_COLS = 800, 96  # the library factors complex64 matrices from this order in blocks of 96 columns
+
+
+def block_update_work(ns, nb=32):
+    """(flops, bytes) of the block updates (k_gemm_tc96) and flops of the updates within the blocks (k_gemm_tc)."""
+    fl = by = inner = 0.0
+    for n in ns:
+        for k0 in range(0, n, BLOCK_COLS):
+            m = n - k0 - BLOCK_COLS
+            if m > 0:
+                fl += 8.0 * BLOCK_COLS * m * m
+                by += 16.0 * m * m + 2 * 8.0 * BLOCK_COLS * m
+            for k in range(k0, min(k0 + BLOCK_COLS, n), nb):
+                cols = min(k0 + BLOCK_COLS, n) - k - nb
+                if cols > 0:
+                    inner += 8.0 * nb * (n - k - nb) * cols
+    return fl, by, inner
+
+
 def kernel_models(K, n_fwd, sweeps, n_delta, n_energy, fp32_ops, fp64_peak, tc_peak, hbm_gbs, precision, nb=32,
-                  sparse=None, solve_cols=0):
+                  sparse=None, bf16_peak=None):
     """Algorithmic real flops per step and the matching peak (TFLOP/s) for each library kernel;
     1 complex multiply-add = 8 real flops.  n_fwd: n of every forward unit; sweeps: per-unit
     refinement sweeps and probes of the forward and of the adjoint."""
@@ -414,32 +433,37 @@ def kernel_models(K, n_fwd, sweeps, n_delta, n_energy, fp32_ops, fp64_peak, tc_p
     df_peak = 8.0 * fp32_ops / DF_OPS_PER_CMAC / 1e12
     m = {}
     ni = [int(x) for x in n_fwd]
-    if mixed:
+    six = bf16_peak / 6.0 if bf16_peak else tc_peak       # six bf16 products per FP32-accurate one
+    fs, fp, bs, bp = sweeps
+    if mixed and max(ni) >= BLOCK_N:
+        fl, by, inner = block_update_work(ni, nb)
+        m["k_gemm_tc96"] = (fl, six, "complex trailing update, 96 columns of L (six bf16 products); peak = measured "
+                            "bf16 / 6", by)
+        m["k_gemm_tc"] = (inner, tc_peak, "updates within the 96-column blocks (3xTF32); peak = measured TF32 / 3")
+    elif mixed:
         m["k_gemm_tc"] = (gemm_flops(ni, nb), tc_peak, "complex trailing update on tcgen05 (3xTF32); peak = "
                           "measured TF32 / 3", gemm_bytes(ni, nb))
     else:
-        m["k_gemm"] = (gemm_flops(ni, nb), simt_peak, "complex trailing update, FP64 DFMA pipe")
-    fs, fp, bs, bp = sweeps
+        m["k_gemm64_tc"] = (gemm_flops(ni, nb), bf16_peak / 28.0 if bf16_peak else simt_peak,
+                            "complex trailing update, exact bf16 digit products; peak = measured bf16 / 28",
+                            2 * gemm_bytes(ni, nb))
     if mixed:
-        rhs = K * (1 + fs) + 2 * K * (1 + bs) + PROBES * (fp + bp)
-        def slices(ncols):  # column slices of a chain solve (the library's rule for solve_cols)
-            if ncols <= 8:
-                return 1
-            sl = solve_cols if solve_cols > 0 else (8 if ncols <= 16 else 16)
-            if sl == 32 and ncols <= 16:
-                sl = 16
-            return -(-ncols // sl)
-        # bytes: one read of the complex64 factors (8 n^2) per unit, column slice and solve
-        reads = slices(K) * (1 + fs) + slices(2 * K) * (1 + bs) + (fp + bp)
-        m["k_solve_c64"] = (float(np.sum(8.0 * n * n * rhs)), simt_peak, "triangular solves (complex64, FP32 pipe)",
-                            float(np.sum(8.0 * n * n * reads)))
+        # bytes: one read of the complex64 factors (8 n^2) per unit and solve
+        m["k_solve_tc"] = (float(np.sum(8.0 * n * n * (K * (1 + fs) + 2 * K * (1 + bs)))), six,
+                           "triangular solves, row products on tcgen05 (six bf16 products); peak = measured bf16 / 6",
+                           float(np.sum(8.0 * n * n * (2 + fs + bs))))
+        m["k_solve_c64"] = (float(np.sum(8.0 * n * n * PROBES * (fp + bp))), simt_peak,
+                            "triangular solves of the convergence probes (2 columns, FP32 pipe)",
+                            float(np.sum(8.0 * n * n * (fp + bp))))
         m["k_residual"] = (float(np.sum(8.0 * n * n * (K * fs + 2 * K * bs))), df_peak,
                            "FP64-accurate residual in double-float FP32 arithmetic (44 FP32 ops per complex MAC)")
         m["k_probe_residual"] = (float(np.sum(8.0 * n * n * PROBES * (fp + bp))), df_peak,
                                  "convergence-probe residual, double-float (2 columns)",
                                  float(np.sum(16.0 * n * n * (fp + bp))))
     else:
-        m["k_solve"] = (float(np.sum(8.0 * n * n * 3.0 * K)), simt_peak, "triangular solves (FP64)")
+        m["k_solve64_tc"] = (float(np.sum(8.0 * n * n * 3.0 * K)), bf16_peak / 36.0 if bf16_peak else simt_peak,
+                             "triangular solves, row products as exact bf16 digit products; peak = measured bf16 / 36",
+                             float(np.sum(16.0 * n * n * 3.0)))
     # assembly: 708 nonzero Gaunt couplings x (complex x real) per off-diagonal block pair (p < q; the
     # block (q, p) is its transpose), once per forward unit
     m["k_assemble"] = (float(np.sum(S * (S - 1) / 2)) * 708 * 4.0, df_peak if mixed else fp64_peak,
@@ -469,7 +493,7 @@ def kernel_rows(kt, models, hbm_gbs):
         if base in models:
             flops, peak, what = models[base][:3]
             ach = flops / (ms * 1e-3) / 1e12
-            row.update({"bound": "tensor" if base == "k_gemm_tc" else "alu", "achieved": ach, "peak": peak,
+            row.update({"bound": "tensor" if "_tc" in base else "alu", "achieved": ach, "peak": peak,
                         "unit": "TFLOP/s", "frac": ach / peak, "work": what})
             if len(models[base]) > 3:  # also HBM-limited: keep whichever roof is closer
                 gbs = models[base][3] / (ms * 1e-3) / 1e9
@@ -677,8 +701,7 @@ def run_ours(args):
     sparse = sparse_product_cmacs(np.asarray(J), np.asarray(w.species), ex["offsets"], ex["site_atom"], grad_sigma,
                                   w.K)
     models = kernel_models(w.K, n_fwd, (fs, fp, bs, bp), w.n_delta, len(w.z), fp32_ops, fp64_peak, tc_peak,
-                           fpk["hbm_gbs"], args.precision, sparse=sparse,
-                           solve_cols=int((tuning or {}).get("solve_cols", 0)))
+                           fpk["hbm_gbs"], args.precision, sparse=sparse, bf16_peak=fpk.get("bf16_tflops"))
     rows = kernel_rows(kt, models, fpk["hbm_gbs"])
     roof = None
     modelled = [r for r in rows.values() if "frac" in r]
