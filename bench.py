@@ -437,20 +437,20 @@ def kernel_models(K, n_fwd, sweeps, n_delta, n_energy, fp32_ops, fp64_peak, tc_p
     fs, fp, bs, bp = sweeps
     if mixed and max(ni) >= BLOCK_N:
         fl, by, inner = block_update_work(ni, nb)
-        m["k_gemm_tc96"] = (fl, six, "complex trailing update, 96 columns of L (six bf16 products); peak = measured "
+        m["k_gemm_tc96"] = (fl, six, "complex trailing update, 96 columns of L (six bf16 products); tensor peak = measured "
                             "bf16 / 6", by)
-        m["k_gemm_tc"] = (inner, tc_peak, "updates within the 96-column blocks (3xTF32); peak = measured TF32 / 3")
+        m["k_gemm_tc"] = (inner, tc_peak, "updates within the 96-column blocks (3xTF32); tensor peak = measured TF32 / 3")
     elif mixed:
         m["k_gemm_tc"] = (gemm_flops(ni, nb), tc_peak, "complex trailing update on tcgen05 (3xTF32); peak = "
                           "measured TF32 / 3", gemm_bytes(ni, nb))
     else:
         m["k_gemm64_tc"] = (gemm_flops(ni, nb), bf16_peak / 28.0 if bf16_peak else simt_peak,
-                            "complex trailing update, exact bf16 digit products; peak = measured bf16 / 28",
+                            "complex trailing update, exact bf16 digit products; tensor peak = measured bf16 / 28",
                             2 * gemm_bytes(ni, nb))
     if mixed:
         # bytes: one read of the complex64 factors (8 n^2) per unit and solve
         m["k_solve_tc"] = (float(np.sum(8.0 * n * n * (K * (1 + fs) + 2 * K * (1 + bs)))), six,
-                           "triangular solves, row products on tcgen05 (six bf16 products); peak = measured bf16 / 6",
+                           "triangular solves, row products on tcgen05 (six bf16 products); tensor peak = measured bf16 / 6",
                            float(np.sum(8.0 * n * n * (2 + fs + bs))))
         m["k_solve_c64"] = (float(np.sum(8.0 * n * n * PROBES * (fp + bp))), simt_peak,
                             "triangular solves of the convergence probes (2 columns, FP32 pipe)",
@@ -462,7 +462,7 @@ def kernel_models(K, n_fwd, sweeps, n_delta, n_energy, fp32_ops, fp64_peak, tc_p
                                  float(np.sum(16.0 * n * n * (fp + bp))))
     else:
         m["k_solve64_tc"] = (float(np.sum(8.0 * n * n * 3.0 * K)), bf16_peak / 36.0 if bf16_peak else simt_peak,
-                             "triangular solves, row products as exact bf16 digit products; peak = measured bf16 / 36",
+                             "triangular solves, row products as exact bf16 digit products; tensor peak = measured bf16 / 36",
                              float(np.sum(16.0 * n * n * 3.0)))
     # assembly: 708 nonzero Gaunt couplings x (complex x real) per off-diagonal block pair (p < q; the
     # block (q, p) is its transpose), once per forward unit
