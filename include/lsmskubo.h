@@ -82,7 +82,9 @@ enum lsms_status {
 };
 
 enum lsms_precision {
-  LSMS_FP64 = 0,   /* plain form: complex128 LU and solves (DFMA) */
+  LSMS_FP64 = 0,   /* plain form: complex128 LU and solves; the row updates as
+                      sums of exact bf16 digit products on the tensor cores
+                      (error as of FP64 arithmetic), the rest in FP64 */
   LSMS_MIXED = 1   /* complex64 LU and solves, FP64 residual and iterative
                       refinement of the tau column block to FP64 accuracy */
 };
