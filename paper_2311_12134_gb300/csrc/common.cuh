@@ -26,6 +26,23 @@ void timer_end(cudaStream_t st);
                           cudaGetErrorString(_e), __FILE__, __LINE__);                   \
   } while (0)
 
+// Opt-in of a kernel to more than 48 KB of dynamic shared memory on the current device.
+template <typename Kernel>
+int smem_limit(SmemLimit& limit, Kernel* kernel, int bytes) {
+  int dev = 0;
+  LSMS_CUDA_TRY(cudaGetDevice(&dev));
+  return limit.raise(dev, bytes, [&]() -> int {
+    LSMS_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    return LSMS_OK;
+  });
+}
+#define LSMS_SMEM_LIMIT(kernel, bytes)                                                  \
+  do {                                                                                   \
+    static ::lsms::SmemLimit _limit;                                                     \
+    const int _rc = ::lsms::smem_limit(_limit, kernel, (int)(bytes));                    \
+    if (_rc) return _rc;                                                                 \
+  } while (0)
+
 // Every kernel launch goes through this: it counts launches and reports a bad
 // launch configuration at once.
 #define LSMS_LAUNCH(kernel, grid, block, smem, stream, ...)                             \

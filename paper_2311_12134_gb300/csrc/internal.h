@@ -2,6 +2,7 @@
 // liblsmskubo.  Not part of the public ABI.
 #pragma once
 
+#include <atomic>
 #include <cstddef>
 #include <cstdint>
 #include <map>
@@ -18,6 +19,28 @@ constexpr int kMaxLmax = 3;
 constexpr int kMaxK = 16;                       // (kMaxLmax + 1)^2
 constexpr int kMaxL3 = 2 * kMaxLmax;            // l'' range of g
 constexpr int kMaxK3 = (kMaxL3 + 1) * (kMaxL3 + 1);
+
+// A kernel's limit of dynamic shared memory.  The runtime keeps it per device and the last value
+// set counts, so each device is told once, and again only for more.  Safe from several host threads.
+class SmemLimit {
+ public:
+  static constexpr int kDevices = 64;
+  // set(): tells the current device dev the new limit; 0 on success
+  template <typename Set>
+  int raise(int dev, int bytes, Set set) {
+    if (dev < 0 || dev >= kDevices) return set();
+    if (limit_[dev].load(std::memory_order_acquire) >= bytes) return LSMS_OK;
+    std::lock_guard<std::mutex> lk(mu_);
+    if (limit_[dev].load(std::memory_order_relaxed) >= bytes) return LSMS_OK;
+    const int rc = set();
+    if (rc == LSMS_OK) limit_[dev].store(bytes, std::memory_order_release);
+    return rc;
+  }
+
+ private:
+  std::mutex mu_;
+  std::atomic<int> limit_[kDevices] = {};
+};
 
 // Error reporting (thread-local message; returns the code for chaining).
 int fail(int code, const char* fmt, ...);

@@ -553,15 +553,9 @@ __global__ void __launch_bounds__(256) k_adj_species(const int32_t* __restrict__
 }
 
 // ------------------------------------------------------------------ wrappers
-static int kubo_partial_attr() {  // more than 48 KB of dynamic shared memory
-  static bool attr_set = false;
-  if (!attr_set) {
-    LSMS_CUDA_TRY(cudaFuncSetAttribute(k_kubo_partial<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)sizeof(KuboShared<true>)));
-    LSMS_CUDA_TRY(cudaFuncSetAttribute(k_kubo_partial<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)sizeof(KuboShared<false>)));
-    attr_set = true;
-  }
+static int kubo_partial_limits() {
+  LSMS_SMEM_LIMIT(k_kubo_partial<true>, sizeof(KuboShared<true>));
+  LSMS_SMEM_LIMIT(k_kubo_partial<false>, sizeof(KuboShared<false>));
   return LSMS_OK;
 }
 
@@ -569,7 +563,7 @@ int kubo_forward(const int64_t* offsets, const int32_t* site_atom, const int32_t
                  const double2* J, int64_t J_dstride, const double2* tau, int64_t S_total, int K, int n_atoms, int n_delta,
                  double volume, bool df, float4* jdf, double2* partial, double2* S, double2* sigma_tilde,
                  double2* sigma, double* rho, cudaStream_t st, int32_t* halve) {
-  const int rc = kubo_partial_attr();
+  const int rc = kubo_partial_limits();
   if (rc) return rc;
   if (halve) {
     const int n_dj = J_dstride > 0 ? n_delta : 1;
@@ -602,7 +596,7 @@ __global__ void k_cscale(double2* __restrict__ x, int64_t n, double a) {
 int kubo_atoms(const int64_t* offsets, const int32_t* site_atom, const int32_t* species, int n_species,
                const double2* J, int64_t J_dstride, const double2* tau, int64_t S_total, int K, int n_atoms,
                int n_delta, double volume, bool df, float4* jdf, double2* out, cudaStream_t st) {
-  const int rc = kubo_partial_attr();
+  const int rc = kubo_partial_limits();
   if (rc) return rc;
   if (df) {
     const int64_t per = (int64_t)n_species * 12 * K * K;

@@ -1467,12 +1467,7 @@ constexpr int kTwoLevelRows = 800;
 template <typename R, int CL>
 static int panel_dsm(const Unit* d_units, int n_units, char* fac_base, int k, int32_t* stat, int m_max, int min_rows,
                      cudaStream_t st) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    LSMS_CUDA_TRY(cudaFuncSetAttribute(k_panel_dsm<R, 32, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       kDsmRows<R> * 32 * (int)sizeof(Cx<R>)));
-    attr_set = true;
-  }
+  LSMS_SMEM_LIMIT((k_panel_dsm<R, 32, CL>), kDsmRows<R> * 32 * sizeof(Cx<R>));
   const int per = (m_max + CL - 1) / CL;
   LSMS_LAUNCH((k_panel_dsm<R, 32, CL>), dim3(CL, n_units), dim3((per + 31) / 32 * 32),
               (size_t)per * 32 * sizeof(Cx<R>), st, d_units, fac_base, k, stat, min_rows);
@@ -1500,17 +1495,10 @@ int lu_factor_chunk(const Unit* d_units, int n_units, int n_max, char* fac_base,
   // rows of a panel that one CTA holds: k_panel_smem (complex64), k_panel_dsm (complex128)
   constexpr int kPanelSmemBytes = 224 * 1024;
   const int max_rows = sizeof(R) == 8 ? kDsmRows<R> : kPanelSmemBytes / (NB * (int)sizeof(Cx<R>));
-  static bool attr_set = false;
-  if (!attr_set) {
-    if constexpr (std::is_same<R, float>::value)
-      LSMS_CUDA_TRY(cudaFuncSetAttribute(k_panel_smem<R, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         kPanelSmemBytes));
-    if (sizeof(Cx<R>) == 8) {
-      LSMS_CUDA_TRY(cudaFuncSetAttribute(k_swap_trsm<R, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         kSwapTileBytes));
-      LSMS_CUDA_TRY(cudaFuncSetAttribute(k_swap_trsm_blk, cudaFuncAttributeMaxDynamicSharedMemorySize, kBlkSmem));
-    }
-    attr_set = true;
+  if constexpr (std::is_same<R, float>::value) {
+    LSMS_SMEM_LIMIT((k_panel_smem<R, NB>), kPanelSmemBytes);
+    LSMS_SMEM_LIMIT((k_swap_trsm<R, NB>), kSwapTileBytes);
+    LSMS_SMEM_LIMIT(k_swap_trsm_blk, kBlkSmem);
   }
   const bool two_level = sizeof(R) == 4 && n_max >= kTwoLevelRows;
   for (int k = 0; k < n_max; k += NB) {
@@ -1589,11 +1577,7 @@ int lu_factor_chunk(const Unit* d_units, int n_units, int n_max, char* fac_base,
     const size_t lap = lap_smem_bytes(n_max);
     if (lap > 227 * 1024 || n_max > kLapMaxN)
       return fail(LSMS_ERR_ARG, "n = %d too large for the complex64 form (at most 16,600)", n_max);
-    static size_t lap_attr = 48 * 1024;
-    if (lap > lap_attr) {
-      LSMS_CUDA_TRY(cudaFuncSetAttribute(k_lapack_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lap));
-      lap_attr = lap;
-    }
+    if (lap > 48 * 1024) LSMS_SMEM_LIMIT(k_lapack_rows, lap);
     const int nb_max = (n_max + 31) / 32;
     if (nb_max > 1)
       LSMS_LAUNCH(k_lapack_rows, dim3((nb_max - 1 + kLapBlocks - 1) / kLapBlocks, n_units), dim3(256), lap, st,
@@ -1657,11 +1641,9 @@ int lu_solve_chunk(const Unit* d_units, int n_units, int n_max, const char* fac_
     if (which_rhs != RHS_X32) return fail(LSMS_ERR_ARG, "internal: complex64 solves work on the X32 field");
     // the right-hand sides in the row order of the factors' permutation
     const size_t pb = (size_t)n_max * sizeof(float2);
-    static size_t perm_attr = 48 * 1024;
-    if (pb > perm_attr) {
+    if (pb > 48 * 1024) {
       if (pb > 227 * 1024) return fail(LSMS_ERR_ARG, "internal: n = %d too large for the permutation", n_max);
-      LSMS_CUDA_TRY(cudaFuncSetAttribute(k_perm_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pb));
-      perm_attr = pb;
+      LSMS_SMEM_LIMIT(k_perm_rows, pb);
     }
     LSMS_LAUNCH(k_perm_rows, dim3(nrhs, n_units), dim3(256), pb, st, d_units, fac_base, ws, nrhs, done);
     const int steps = solve_path(n_units, n_max);

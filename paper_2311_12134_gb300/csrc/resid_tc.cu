@@ -408,12 +408,7 @@ __global__ void __launch_bounds__(256, 2) k_residual_tc(const Unit* __restrict__
 
 int residual_tc_chunk(const Unit* d_units, int n_units, int n_max, const char* fac_base, char* ws, int K, int nrhs,
                       bool explicit_b, const int32_t* done, int32_t* stat, cudaStream_t st) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    LSMS_CUDA_TRY(cudaFuncSetAttribute(k_residual_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       rtc::SMEM_LAUNCH));
-    attr_set = true;
-  }
+  LSMS_SMEM_LIMIT(k_residual_tc, rtc::SMEM_LAUNCH);
   const dim3 grid((n_max + rtc::TM - 1) / rtc::TM, n_units, (nrhs + rtc::NC - 1) / rtc::NC);
   LSMS_LAUNCH(k_residual_tc, grid, dim3(rtc::NT), rtc::SMEM_LAUNCH, st, d_units, fac_base, ws, K, nrhs, explicit_b,
               done, stat);

@@ -336,11 +336,7 @@ __global__ void __launch_bounds__(128) k_gemm_tc(const Unit* __restrict__ units,
 
 int gemm_tc_chunk(const Unit* d_units, int n_units, int n_max, int k, int c_end, char* fac_base, int32_t* stat,
                   cudaStream_t st) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    LSMS_CUDA_TRY(cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_BYTES));
-    attr_set = true;
-  }
+  LSMS_SMEM_LIMIT(k_gemm_tc, tc::SMEM_BYTES);
   const int mt = n_max - k - tc::NB;
   if (mt <= 0) return LSMS_OK;
   const int tm = (mt + tc::TM - 1) / tc::TM;
@@ -538,11 +534,7 @@ __global__ void __launch_bounds__(128) k_step_tc(const Unit* __restrict__ units,
 
 int step_tc_chunk(const Unit* d_units, int n_units, int n_max, const char* fac_base, char* ws, int nrhs,
                   const int32_t* done, int32_t* stat, int s, bool forward, cudaStream_t st) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    LSMS_CUDA_TRY(cudaFuncSetAttribute(k_step_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_BYTES));
-    attr_set = true;
-  }
+  LSMS_SMEM_LIMIT(k_step_tc, tc::SMEM_BYTES);
   if (nrhs < 1 || nrhs > tc::TNC) return fail(LSMS_ERR_ARG, "internal: step_tc_chunk nrhs %d", nrhs);
   const int rows = forward ? n_max - tc::NB * (s + 1) : tc::NB * s;
   if (rows <= 0) return LSMS_OK;

@@ -359,12 +359,7 @@ __global__ void __launch_bounds__(oz::NT, 1) k_gemm64_tc(const Unit* __restrict_
 
 int gemm64_tc_chunk(const Unit* d_units, int n_units, int n_max, int k, char* fac_base, int32_t* stat,
                     cudaStream_t st) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    LSMS_CUDA_TRY(cudaFuncSetAttribute(k_gemm64_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       oz::kGemmSmem));
-    attr_set = true;
-  }
+  LSMS_SMEM_LIMIT(k_gemm64_tc, oz::kGemmSmem);
   const int mt = n_max - k - oz::NB;
   if (mt <= 0) return LSMS_OK;
   const int rows = (mt + oz::TM - 1) / oz::TM, tiles = (mt + oz::NCC - 1) / oz::NCC;
@@ -700,12 +695,7 @@ __global__ void __launch_bounds__(oz::NT, 1) k_solve64_tc(const Unit* __restrict
 
 int solve64_tc_chunk(const Unit* d_units, int n_units, const char* fac_base, char* ws, int nrhs, int32_t* stat,
                      cudaStream_t st) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    LSMS_CUDA_TRY(cudaFuncSetAttribute(k_solve64_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       oz::kSolveSmem));
-    attr_set = true;
-  }
+  LSMS_SMEM_LIMIT(k_solve64_tc, oz::kSolveSmem);
   LSMS_LAUNCH(k_solve64_tc, dim3(n_units, (nrhs + oz::NCC - 1) / oz::NCC), dim3(oz::NT),
               oz::kSolveSmem, st, d_units,
               fac_base, ws, nrhs, stat);

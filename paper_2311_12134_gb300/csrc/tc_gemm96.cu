@@ -278,11 +278,7 @@ __global__ void __launch_bounds__(tg::NT, 1) k_gemm_tc96(const Unit* __restrict_
 
 int gemm_tc96_chunk(const Unit* d_units, int n_units, int n_max, int K0, char* fac_base, int32_t* stat,
                      cudaStream_t st) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    LSMS_CUDA_TRY(cudaFuncSetAttribute(k_gemm_tc96, cudaFuncAttributeMaxDynamicSharedMemorySize, tg::SMEM_BYTES));
-    attr_set = true;
-  }
+  LSMS_SMEM_LIMIT(k_gemm_tc96, tg::SMEM_BYTES);
   const int mt = n_max - K0 - tg::KB;
   if (mt <= 0) return LSMS_OK;
   const int rows = (mt + tg::TM - 1) / tg::TM, tiles = (mt + tg::NCC - 1) / tg::NCC;

@@ -392,12 +392,8 @@ __global__ void __launch_bounds__(ts::NT, 2) k_solve_tc(const Unit* __restrict__
 
 int solve_tc_chunk(const Unit* d_units, int n_units, const char* fac_base, char* ws, int nrhs, const int32_t* done,
                    int32_t* stat, cudaStream_t st) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    LSMS_CUDA_TRY(cudaFuncSetAttribute(k_solve_tc<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, ts::kSmem<16>));
-    LSMS_CUDA_TRY(cudaFuncSetAttribute(k_solve_tc<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, ts::kSmem<32>));
-    attr_set = true;
-  }
+  LSMS_SMEM_LIMIT(k_solve_tc<16>, ts::kSmem<16>);
+  LSMS_SMEM_LIMIT(k_solve_tc<32>, ts::kSmem<32>);
   if (nrhs < 1 || nrhs > 32) return fail(LSMS_ERR_ARG, "internal: solve_tc_chunk nrhs %d", nrhs);
   if (nrhs <= 16)
     LSMS_LAUNCH(k_solve_tc<16>, dim3(n_units), dim3(ts::NT), ts::kSmem<16>, st, d_units, fac_base, ws, nrhs, done, stat);
