@@ -1543,11 +1543,11 @@ static int solve_refine(const Call& c, const Plan& p, const Chunk& ch, const cha
   if (c.precision == LSMS_FP64) {
     if (explicit_b) LSMS_LAUNCH(k_copy_b, g1, dim3(256), 0, c.st, du, ws, nrhs, false);
     else LSMS_LAUNCH(k_rhs_identity<double2>, g1, dim3(256), 0, c.st, du, ws, (int)RHS_X, c.K, nrhs);
-    return lu_solve_chunk<double>(du, nu, ch.n_max, fac_base, ws, RHS_X, nrhs, nullptr, stat, c.st);
+    return lu_solve_chunk<double>(du, nu, ch.n_max, fac_base, ws, RHS_X, nrhs, nullptr, ch.path, stat, c.st);
   }
   if (explicit_b) LSMS_LAUNCH(k_copy_b, g1, dim3(256), 0, c.st, du, ws, nrhs, true);
   else LSMS_LAUNCH(k_rhs_identity<float2>, g1, dim3(256), 0, c.st, du, ws, (int)RHS_X32, c.K, nrhs);
-  if ((rc = lu_solve_chunk<float>(du, nu, ch.n_max, fac_base, ws, RHS_X32, nrhs, nullptr, stat, c.st))) return rc;
+  if ((rc = lu_solve_chunk<float>(du, nu, ch.n_max, fac_base, ws, RHS_X32, nrhs, nullptr, ch.path, stat, c.st))) return rc;
   LSMS_LAUNCH(k_widen, dim3(nu), dim3(256), 0, c.st, du, ws, nrhs);
   // done flags of this chunk's units start cleared (memset by the caller)
   const int max_sweeps = opt_ir_max_sweeps();
@@ -1568,12 +1568,12 @@ static int solve_refine(const Call& c, const Plan& p, const Chunk& ch, const cha
 #undef LSMS_RESID
       default: return fail(LSMS_ERR_ARG, "internal: no residual kernel for %d right-hand sides", nrhs);
     }
-    if ((rc = lu_solve_chunk<float>(du, nu, ch.n_max, fac_base, ws, RHS_X32, nrhs, done, stat, c.st))) return rc;
+    if ((rc = lu_solve_chunk<float>(du, nu, ch.n_max, fac_base, ws, RHS_X32, nrhs, done, ch.path, stat, c.st))) return rc;
     LSMS_LAUNCH(k_ir_update, dim3(nu), dim3(256), 0, c.st, du, ws, nrhs, c.K, explicit_b, it, kIrTol, done,
                 stat);
     // probe: would the next sweep's correction pass the test?  If so, stop here.
     LSMS_LAUNCH(k_probe_residual, gr, dim3(256), 0, c.st, du, fac_base, ws, done);
-    if ((rc = lu_solve_chunk<float>(du, nu, ch.n_max, fac_base, ws, RHS_X32, kProbe, done, stat, c.st))) return rc;
+    if ((rc = lu_solve_chunk<float>(du, nu, ch.n_max, fac_base, ws, RHS_X32, kProbe, done, ch.path, stat, c.st))) return rc;
     LSMS_LAUNCH(k_probe_check, dim3(nu), dim3(256), 0, c.st, du, ws, kIrTol, done, stat);
   }
   LSMS_LAUNCH(k_ir_finish, dim3((nu + 255) / 256), dim3(256), 0, c.st, du, nu, done, stat);
@@ -1615,7 +1615,7 @@ static int fallback_resolve(const Call& c, const Plan& p, char* ws, const WsHead
   const dim3 g1((n_max * nrhs + 255) / 256, slots);
   if (!adj) {
     LSMS_LAUNCH(k_rhs_identity<double2>, g1, dim3(256), 0, c.st, fbu, region, (int)RHS_X, c.K, nrhs);
-    if ((rc = lu_solve_chunk<double>(fbu, slots, n_max, region, region, RHS_X, nrhs, nullptr, stat, c.st))) return rc;
+    if ((rc = lu_solve_chunk<double>(fbu, slots, n_max, region, region, RHS_X, nrhs, nullptr, 1, stat, c.st))) return rc;
     LSMS_LAUNCH(k_write_tau, dim3(S_max, slots), dim3(256), 0, c.st, fbu, region, c.K, c.liz->total_sites, c.conj,
                 tau_out);
     return LSMS_OK;
@@ -1624,7 +1624,7 @@ static int fallback_resolve(const Call& c, const Plan& p, char* ws, const WsHead
                     c.liz->total_sites, adj->abar, nullptr, 0, nullptr, adj->n_delta, c.K, region, false, c.st)))
     return rc;
   LSMS_LAUNCH(k_copy_b, g1, dim3(256), 0, c.st, fbu, region, nrhs, false);
-  if ((rc = lu_solve_chunk<double>(fbu, slots, n_max, region, region, RHS_X, nrhs, nullptr, stat, c.st))) return rc;
+  if ((rc = lu_solve_chunk<double>(fbu, slots, n_max, region, region, RHS_X, nrhs, nullptr, 1, stat, c.st))) return rc;
   return adj_site(fbu, slots, S_max, adj->tau, c.liz->total_sites, c.K, region, adj->G, false, c.st);
 }
 
@@ -1667,16 +1667,17 @@ static int asked_parts() {
 //    3.16 and 3.67; from 216 units of n = 880 on four parts gain (18.7 and 17.8 ms);
 //  - where the solves run as block-step launches: a part's thousands of launches fill the launch
 //    queue before the next part's first one is enqueued, so parts run one after the other, each on a
-//    nearly idle GPU (54 atoms of n = 2192 90 ms in one part, 155 in four; 2 of n = 15,440 970 and
-//    1296 in two).
+//    nearly idle GPU (2 atoms of n = 15,440 970 ms in one part, 1296 in two).  The path is that of
+//    the whole chunk (ch.path): asked anew for each part, a chunk of a little over n / 64 units was
+//    cut in four for its chains and each part then took block steps (108 units of n = 4144 438 ms
+//    per step; chains in four parts 289, in one 282).
 static int parts_of(const Plan& p, const Chunk& ch) {
   const int asked = asked_parts();
   if (asked) return asked;
   int64_t rows = 0;
   for (int f = ch.f0; f < ch.f1; ++f) rows += p.fac_units[f].n;
   if (rows < 65536) return 1;
-  if (p.precision == LSMS_MIXED && solve_path(ch.u1 - ch.u0, ch.n_max) != 1) return 1;
-  return kMaxParts;
+  return ch.path != 1 ? 1 : kMaxParts;
 }
 
 static int side_streams(SideStreams** out) {
@@ -1719,8 +1720,9 @@ static int split_chunk(const Plan& p, const Chunk& ch, int want, Chunk* part) {
 
 // run(chunk, stream) for the parts of ch on concurrent streams, or for ch on c.st.
 template <typename F>
-static int run_split(const Call& c, const Plan& p, const Chunk& ch, F run) {
-  Chunk part[kMaxParts];
+static int run_split(const Call& c, const Plan& p, const Chunk& chunk, F run) {
+  Chunk ch = chunk, part[kMaxParts];
+  if (p.precision == LSMS_MIXED) ch.path = solve_path(ch.u1 - ch.u0, ch.n_max);
   const int np = g_timer_on.load(std::memory_order_relaxed) ? 1 : split_chunk(p, ch, parts_of(p, ch), part);
   if (np == 1) return run(ch, c.st);
   SideStreams* ss = nullptr;

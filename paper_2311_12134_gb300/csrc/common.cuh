@@ -272,10 +272,11 @@ template <typename R>
 int lu_factor_chunk(const Unit* d_units, int n_units, int n_max, char* fac_base,
                     int32_t* stat, cudaStream_t st);
 // Solve L U X = P B in place for the n x nrhs column-major block at
-// ws + unit.<field> (complex<R>), skipping units whose done flag is set.
+// ws + unit.<field> (complex<R>), skipping units whose done flag is set.  path: how the
+// complex64 solves run (solve_path).
 template <typename R>
 int lu_solve_chunk(const Unit* d_units, int n_units, int n_max, const char* fac_base, char* ws,
-                   int which_rhs, int nrhs, const int32_t* done, int32_t* stat, cudaStream_t st);
+                   int which_rhs, int nrhs, const int32_t* done, int path, int32_t* stat, cudaStream_t st);
 
 enum RhsField { RHS_X = 0, RHS_X32 = 1 };
 

@@ -99,6 +99,7 @@ struct Chunk {
   int f0, f1;        // range of the units that own factors (fac_units)
   int n_max;         // largest n in the chunk (units are sorted by n, descending)
   size_t ws_bytes;   // workspace bytes used by the chunk
+  int path = 1;      // complex64 solves (solve_path), decided for the whole chunk and kept by its parts
 };
 
 // Work plan of one call shape.  units: every (atom, energy) system solved;

@@ -1634,7 +1634,7 @@ int solve_path(int n_units, int n_max) {
 
 template <typename R>
 int lu_solve_chunk(const Unit* d_units, int n_units, int n_max, const char* fac_base, char* ws, int which_rhs,
-                   int nrhs, const int32_t* done, int32_t* stat, cudaStream_t st) {
+                   int nrhs, const int32_t* done, int path, int32_t* stat, cudaStream_t st) {
   if (nrhs < 1 || nrhs > 32) return fail(LSMS_ERR_ARG, "internal: nrhs %d out of range", nrhs);
   constexpr int NB = LuCfg<R>::NB;
   if constexpr (std::is_same<R, float>::value) {
@@ -1646,9 +1646,8 @@ int lu_solve_chunk(const Unit* d_units, int n_units, int n_max, const char* fac_
       LSMS_SMEM_LIMIT(k_perm_rows, pb);
     }
     LSMS_LAUNCH(k_perm_rows, dim3(nrhs, n_units), dim3(256), pb, st, d_units, fac_base, ws, nrhs, done);
-    const int steps = solve_path(n_units, n_max);
-    if (steps == 3) return solve_steps_tc(d_units, n_units, n_max, fac_base, ws, nrhs, done, stat, st);
-    if (steps == 2) {
+    if (path == 3) return solve_steps_tc(d_units, n_units, n_max, fac_base, ws, nrhs, done, stat, st);
+    if (path == 2) {
       if (nrhs <= 8) return solve_steps<8>(d_units, n_units, n_max, fac_base, ws, nrhs, done, st);
       if (nrhs <= 16) return solve_steps<16>(d_units, n_units, n_max, fac_base, ws, nrhs, done, st);
       return solve_steps<32>(d_units, n_units, n_max, fac_base, ws, nrhs, done, st);
@@ -1667,9 +1666,9 @@ int lu_solve_chunk(const Unit* d_units, int n_units, int n_max, const char* fac_
 
 template int lu_factor_chunk<double>(const Unit*, int, int, char*, int32_t*, cudaStream_t);
 template int lu_factor_chunk<float>(const Unit*, int, int, char*, int32_t*, cudaStream_t);
-template int lu_solve_chunk<double>(const Unit*, int, int, const char*, char*, int, int, const int32_t*, int32_t*,
+template int lu_solve_chunk<double>(const Unit*, int, int, const char*, char*, int, int, const int32_t*, int, int32_t*,
                                     cudaStream_t);
-template int lu_solve_chunk<float>(const Unit*, int, int, const char*, char*, int, int, const int32_t*, int32_t*,
+template int lu_solve_chunk<float>(const Unit*, int, int, const char*, char*, int, int, const int32_t*, int, int32_t*,
                                    cudaStream_t);
 
 }  // namespace lsms
