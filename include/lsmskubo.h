@@ -335,9 +335,9 @@ int lsms_kubo_sigma_backward(const lsms_liz* liz, int lmax, const int32_t* speci
  *                     0 disables the fallback); enters the workspace sizes
  *   "ir_max_sweeps"   refinement sweeps of the mixed form before
  *                     LSMS_UNIT_NOCONV (default 6; 0..64)
- *   "streams"         concurrent parts per chunk (1..4; 0 = the environment
- *                     variable LSMS_STREAMS, else 4, or 1 for small chunks and
- *                     where the solves run as block steps)
+ *   "streams"         concurrent parts per chunk (1..4; 0 (default) = the
+ *                     environment variable LSMS_STREAMS, else 4, or 1 for small
+ *                     chunks and where the solves run as block steps)
  *   "residual_tc"     1 (default): the mixed form's refinement residual for 9
  *                     or more right-hand sides runs on the tensor cores (bf16
  *                     fixed-point digits, exact FP32 accumulation, about 2^-48
@@ -355,8 +355,9 @@ int lsms_kubo_sigma_backward(const lsms_liz* liz, int lmax, const int32_t* speci
  *                     CTAs on the FP32 pipes; 3: the same with the row updates as
  *                     3xTF32 products on the tensor cores; 0 (default): chains,
  *                     but block steps (2) for few units of large matrices
- *                     (n >= 3000 and at most n / 64 units in a chunk part)
- * LSMS_ERR_ARG for an unknown name or a value out of range. */
+ *                     (n >= 3000 and at most n / 64 units in a chunk)
+ * lsms_get_option gives the value set, or the default.  LSMS_ERR_ARG for an
+ * unknown name or a value out of range. */
 int lsms_set_option(const char* name, double value);
 int lsms_get_option(const char* name, double* value);
 

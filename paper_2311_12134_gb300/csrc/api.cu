@@ -1802,7 +1802,7 @@ extern "C" int lsms_get_option(const char* name, double* value) {
   if (n == "growth_limit") *value = g_opt_growth_limit.load();
   else if (n == "fallback_slots") *value = g_opt_fallback_slots.load();
   else if (n == "ir_max_sweeps") *value = g_opt_ir_max_sweeps.load();
-  else if (n == "streams") *value = asked_parts() ? asked_parts() : kMaxParts;
+  else if (n == "streams") *value = g_opt_streams.load();
   else if (n == "residual_tc") *value = g_opt_residual_tc.load();
   else if (n == "solve_cols") *value = g_opt_solve_cols.load();
   else if (n == "solve_regs") *value = g_opt_solve_regs.load();
