@@ -32,11 +32,23 @@ def check_unit_status(status):
     return st
 
 
-# Adjoint workspace when the caller gave no cap (the library's own default chunk budget).  Sized as
-# the forward's, which holds only right-hand sides when the factors are kept, the adjoint ran in
-# chunks of few units: 108 chunks and 243 ms per step for 108 atoms of n = 880 (conjugate pairs), 32
-# chunks and 17 ms for the 32-atom FP64 step; in one chunk 18.6 and 4.0 ms.
-ADJOINT_CHUNK_BYTES = 8 << 30
+# Adjoint workspace when the caller gave no cap.  Sized as the forward's, which holds only
+# right-hand sides when the factors are kept, the adjoint ran in chunks of few units: 243 ms per step
+# for 108 atoms of n = 880 (conjugate pairs, 161 MB), 16 for the 32-atom FP64 step (7 MB); in one chunk
+# 16.4 ms (494 MB) and 3.3 (19 MB).  From some 300 units in a chunk on nothing is gained: 1,488 units of
+# n about 850 take 105.7 ms with 945 MB and 105.8 with 2,696, 6,084 units 434 ms with 3.6 GB or 8.  So
+# it grows by 2 GiB at most (n = 4144, 108 units: 2.4 to 3.0 GB, 381 to 290 ms), and a Problem that is
+# not alone on the device, or close to the end of its memory, keeps the small one: the growth takes at
+# most 1 / ADJOINT_FREE_SHARE of what is free.
+ADJOINT_GROWTH_BYTES = 2 << 30
+ADJOINT_FREE_SHARE = 16
+
+
+def _free_bytes(device):
+    """Device memory that PyTorch can still hand out: free on the device, or cached and unused."""
+    import torch
+    cached = torch.cuda.memory_reserved(device) - torch.cuda.memory_allocated(device)
+    return torch.cuda.mem_get_info(device)[0] + cached
 
 
 class Problem:
@@ -161,10 +173,12 @@ class Problem:
 
     def _adjoint_workspace(self, mn, al):
         """Workspace of the adjoint, between the sizes for one atom and for all units: as large as the
-        forward's; without a cap from the caller, up to ADJOINT_CHUNK_BYTES where the memory is there."""
+        forward's; without a cap from the caller, up to ADJOINT_GROWTH_BYTES more where the memory is there."""
         import torch
         small = min(al, max(mn, self.workspace.numel()))
-        size = small if self._capped else min(al, max(small, ADJOINT_CHUNK_BYTES))
+        size = small if self._capped else min(al, small + ADJOINT_GROWTH_BYTES)
+        if size > small and (size - small) * ADJOINT_FREE_SHARE > _free_bytes(self.device):
+            size = small
         try:
             return torch.empty(size, dtype=torch.uint8, device=self.device)
         except torch.OutOfMemoryError:
