@@ -41,6 +41,7 @@ def check_unit_status(status):
 # not alone on the device, or close to the end of its memory, keeps the small one: the growth takes at
 # most 1 / ADJOINT_FREE_SHARE of what is free.
 ADJOINT_GROWTH_BYTES = 2 << 30
+DETACHED_GROWTH_BYTES = 8 << 30  # with the factors in it and given back at once: the library's own chunk budget
 ADJOINT_FREE_SHARE = 16
 
 
@@ -171,12 +172,12 @@ class Problem:
         grad_tinv_species))."""
         return _step(self, grad_sigma, tinv)
 
-    def _adjoint_workspace(self, mn, al):
+    def _adjoint_workspace(self, mn, al, growth=ADJOINT_GROWTH_BYTES):
         """Workspace of the adjoint, between the sizes for one atom and for all units: as large as the
-        forward's; without a cap from the caller, up to ADJOINT_GROWTH_BYTES more where the memory is there."""
+        forward's; without a cap from the caller, up to `growth` bytes more where the memory is there."""
         import torch
         small = min(al, max(mn, self.workspace.numel()))
-        size = small if self._capped else min(al, small + ADJOINT_GROWTH_BYTES)
+        size = small if self._capped else min(al, small + growth)
         if size > small and (size - small) * ADJOINT_FREE_SHARE > _free_bytes(self.device):
             size = small
         try:
@@ -216,7 +217,7 @@ class Problem:
         self._maybe_check(st)
         del ws
         mn, al = B.backward_workspace_bytes(self.liz, self.lmax, nE, prec)
-        bws = self._adjoint_workspace(mn, al)
+        bws = self._adjoint_workspace(mn, al, DETACHED_GROWTH_BYTES)
         bst = torch.empty_like(self.bw_status)
         out = B.kubo_sigma_backward(self.liz, self.lmax, self.species, tinv, self.z, self.J, tau, self.volume,
                                     grad_sigma.contiguous(), self.precision, lu_store=None, unit_status=bst,
