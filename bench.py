@@ -202,7 +202,7 @@ def gemm_flops(n_list, nb):
 
 
 def file_peaks():
-    """Measured peaks of this GPU pool (MEASURED_PEAKS.json), else the fallback figures."""
+    """Measured peaks of the GPU (MEASURED_PEAKS.json), else the fallback figures."""
     p = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustained": 1700.0, "sm_max_mhz": 2070.0,
          "source": "fallback"}
     path = os.path.join(ROOT, "MEASURED_PEAKS.json")
@@ -402,12 +402,15 @@ def sparse_product_cmacs(J, species, offsets, site_atom, weights, K):
     return adj, trace
 
 
-BLOCK_N, BLOCK_COLS = 800, 96  # the library factors complex64 matrices from this order in blocks of 96 columns
+# The library factors complex64 matrices from this order in blocks of 96 columns (kTwoLevelRows and kBlkK of its
+# sources).  It decides by the largest order of a chunk part, here by each unit's: parts hold units sorted by
+# order, so only the smaller units of the one part in which the line lies are counted to the other update.
+BLOCK_N, BLOCK_COLS = 800, 96
 
 
 def block_update_work(ns, nb=32):
-    """(flops, bytes) of the block updates (k_gemm_tc96) and flops of the updates within the blocks (k_gemm_tc)."""
-    fl = by = inner = 0.0
+    """(flops, bytes) of the block updates (k_gemm_tc96), then of the updates within the blocks (k_gemm_tc)."""
+    fl = by = inner = inner_by = 0.0
     for n in ns:
         for k0 in range(0, n, BLOCK_COLS):
             m = n - k0 - BLOCK_COLS
@@ -417,8 +420,10 @@ def block_update_work(ns, nb=32):
             for k in range(k0, min(k0 + BLOCK_COLS, n), nb):
                 cols = min(k0 + BLOCK_COLS, n) - k - nb
                 if cols > 0:
-                    inner += 8.0 * nb * (n - k - nb) * cols
-    return fl, by, inner
+                    rows = n - k - nb
+                    inner += 8.0 * nb * rows * cols
+                    inner_by += 16.0 * rows * cols + 8.0 * nb * (rows + cols)
+    return fl, by, inner, inner_by
 
 
 def kernel_models(K, n_fwd, sweeps, n_delta, n_energy, fp32_ops, fp64_peak, tc_peak, hbm_gbs, precision, nb=32,
@@ -435,17 +440,18 @@ def kernel_models(K, n_fwd, sweeps, n_delta, n_energy, fp32_ops, fp64_peak, tc_p
     ni = [int(x) for x in n_fwd]
     six = bf16_peak / 6.0 if bf16_peak else tc_peak       # six bf16 products per FP32-accurate one
     fs, fp, bs, bp = sweeps
-    if mixed and max(ni) >= BLOCK_N:
-        fl, by, inner = block_update_work(ni, nb)
-        m["k_gemm_tc96"] = (fl, six, "complex trailing update, 96 columns of L (six bf16 products); tensor peak = measured "
-                            "bf16 / 6", by)
-        m["k_gemm_tc"] = (inner, tc_peak, "updates within the 96-column blocks (3xTF32); tensor peak = measured TF32 / 3")
-    elif mixed:
-        m["k_gemm_tc"] = (gemm_flops(ni, nb), tc_peak, "complex trailing update on tcgen05 (3xTF32); peak = "
-                          "measured TF32 / 3", gemm_bytes(ni, nb))
+    if mixed:
+        small = [x for x in ni if x < BLOCK_N]
+        fl, by, inner, inner_by = block_update_work([x for x in ni if x >= BLOCK_N], nb)
+        if fl:
+            m["k_gemm_tc96"] = (fl, six, "complex trailing update, 96 columns of L (six bf16 products); tensor peak = "
+                                "measured bf16 / 6", by)
+        m["k_gemm_tc"] = (inner + gemm_flops(small, nb), tc_peak, "complex trailing update, 32 columns of L, and updates "
+                          "within the 96-column blocks (3xTF32); tensor peak = measured TF32 / 3",
+                          inner_by + gemm_bytes(small, nb))
     else:
-        m["k_gemm64_tc"] = (gemm_flops(ni, nb), bf16_peak / 28.0 if bf16_peak else simt_peak,
-                            "complex trailing update, exact bf16 digit products; tensor peak = measured bf16 / 28",
+        m["k_gemm64_tc"] = (gemm_flops(ni, nb), bf16_peak / 34.0 if bf16_peak else simt_peak,
+                            "complex trailing update, exact bf16 digit products; tensor peak = measured bf16 / 34",
                             2 * gemm_bytes(ni, nb))
     if mixed:
         # bytes: one read of the complex64 factors (8 n^2) per unit and solve
@@ -461,8 +467,8 @@ def kernel_models(K, n_fwd, sweeps, n_delta, n_energy, fp32_ops, fp64_peak, tc_p
                                  "convergence-probe residual, double-float (2 columns)",
                                  float(np.sum(16.0 * n * n * (fp + bp))))
     else:
-        m["k_solve64_tc"] = (float(np.sum(8.0 * n * n * 3.0 * K)), bf16_peak / 36.0 if bf16_peak else simt_peak,
-                             "triangular solves, row products as exact bf16 digit products; tensor peak = measured bf16 / 36",
+        m["k_solve64_tc"] = (float(np.sum(8.0 * n * n * 3.0 * K)), bf16_peak / 34.0 if bf16_peak else simt_peak,
+                             "triangular solves, row products as exact bf16 digit products; tensor peak = measured bf16 / 34",
                              float(np.sum(16.0 * n * n * 3.0)))
     # assembly: 708 nonzero Gaunt couplings x (complex x real) per off-diagonal block pair (p < q; the
     # block (q, p) is its transpose), once per forward unit
