@@ -39,10 +39,12 @@ def check_unit_status(status):
 # n about 850 take 105.7 ms with 945 MB and 105.8 with 2,696, 6,084 units 434 ms with 3.6 GB or 8.  So
 # it grows by 2 GiB at most (n = 4144, 108 units: 2.4 to 3.0 GB, 381 to 290 ms), and a Problem that is
 # not alone on the device, or close to the end of its memory, keeps the small one: the growth takes at
-# most 1 / ADJOINT_FREE_SHARE of what is free.
+# most 1 / ADJOINT_FREE_SHARE of what is free (asked for above ADJOINT_ASK_BYTES: the question takes 0.2 ms
+# of a first pass of 2.7).
 ADJOINT_GROWTH_BYTES = 2 << 30
 DETACHED_GROWTH_BYTES = 8 << 30  # with the factors in it and given back at once: the library's own chunk budget
 ADJOINT_FREE_SHARE = 16
+ADJOINT_ASK_BYTES = 64 << 20
 
 
 def _free_bytes(device):
@@ -178,7 +180,7 @@ class Problem:
         import torch
         small = min(al, max(mn, self.workspace.numel()))
         size = small if self._capped else min(al, small + growth)
-        if size > small and (size - small) * ADJOINT_FREE_SHARE > _free_bytes(self.device):
+        if size - small > ADJOINT_ASK_BYTES and (size - small) * ADJOINT_FREE_SHARE > _free_bytes(self.device):
             size = small
         try:
             return torch.empty(size, dtype=torch.uint8, device=self.device)

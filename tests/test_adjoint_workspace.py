@@ -33,3 +33,5 @@ def test_adjoint_workspace_leaves_the_rest_of_a_full_device(monkeypatch):
     assert _size(monkeypatch, 160 * MB, 161 * MB, 494 * MB, 4 * GB) == 161 * MB
     assert _size(monkeypatch, 160 * MB, 161 * MB, 494 * MB, 1 * GB, cached=20 * GB) == 494 * MB
     assert _size(monkeypatch, 3 * MB, 7 * MB, 19 * MB, 4 * GB) == 19 * MB
+    assert _size(monkeypatch, 3 * MB, 7 * MB, 71 * MB, 0) == 71 * MB  # 64 MB are taken without asking
+    assert _size(monkeypatch, 3 * MB, 7 * MB, 72 * MB, 0) == 7 * MB
