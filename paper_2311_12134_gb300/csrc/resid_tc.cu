@@ -6,17 +6,16 @@
 // row's largest |Re| or |Im|, recorded by the assembly), column c of X by
 // 2^-F_c (recorded by k_widen / k_ir_update).  Each scaled real value, held as a
 // double-float pair, becomes six balanced base-256 digits
-//   v 2^7 = sum_{s=1..6} a_s 2^{8 (1 - s)} + rest,  a_s integers, |a_s| <= 129,
-//   |rest| <= 2^-41 (2^-48 of the scale),
-// all exact in bf16.  A digit product a_s b_t is an integer of at most 129^2 and
-// belongs to weight class g = s + t; the 21 pairs with g <= 7 run as bf16
-// tcgen05.mma with FP32 accumulation in tensor memory, one accumulator per class.
-// Per real K a class sum grows by at most 6 * 129^2 < 2^17, so 128 real K
-// accumulate exactly in FP32 (below 2^24): every 4 chunks of 32 real K the
-// accumulators are read with tcgen05.ld and added, scaled by 2^{-8 (g - 2)},
-// into double-float registers.  The dropped classes (g >= 8) and the digit
-// rests stay below 2^-48 of the scales.  The complex product is the real
-// embedding
+//   v 2^7 = sum_{s=1..6} a_s 2^{8 (1 - s)} + rest,  |rest| <= 2^-41 (2^-48 of the scale),
+//   a_s integers, |a_s| <= 128 for s <= 3, 192 for s = 4, 129 for s = 5 and 6 (digits6x2),
+// all exact in bf16.  A digit product a_s b_t is an integer of weight class g = s + t;
+// the 21 pairs with g <= 7 run as bf16 tcgen05.mma with FP32 accumulation in tensor
+// memory, one accumulator per class.  Per real K a class sum grows by at most
+// 4 * 128 * 129 + 2 * 128 * 192 < 2^17 (g = 7), so 128 real K accumulate exactly in FP32
+// (below 2^24): every 4 chunks of 32 real K the accumulators are read with tcgen05.ld and
+// added, scaled by 2^{-8 (g - 2)}, into double-float registers.  The dropped classes
+// (g >= 8) and the digit rests stay below 2^-48 of the scales.  The complex product is the
+// real embedding
 //   [Re MX | Im MX] = [Re M | Im M] x [[Re X, Im X], [-Im X, Re X]].
 //
 // CTA: 128 rows of one unit (TMEM lanes), 16 complex right-hand-side columns

@@ -1,6 +1,6 @@
 """The size of the adjoint's workspace (kept by a Problem for its lifetime): all units where that is little,
-at most 2 GiB more than the forward's, and the forward's size where the growth would take more than a
-sixteenth of the free memory or the caller gave a cap.  Host only: the device's free memory is made up."""
+at most 2 GiB more than the forward's, and the forward's size where the growth is above 64 MiB and more than
+a sixteenth of the free memory, or the caller gave a cap.  Host only: the device's free memory is made up."""
 import types
 
 import pytest
