@@ -402,10 +402,19 @@ def sparse_product_cmacs(J, species, offsets, site_atom, weights, K):
     return adj, trace
 
 
-# The library factors complex64 matrices from this order in blocks of 96 columns (kTwoLevelRows and kBlkK of its
-# sources).  It decides by the largest order of a chunk part, here by each unit's: parts hold units sorted by
-# order, so only the smaller units of the one part in which the line lies are counted to the other update.
+# The library factors complex64 matrices in blocks of 96 columns where the largest order of a chunk part is
+# at least this (kTwoLevelRows and kBlkK of its sources).
 BLOCK_N, BLOCK_COLS = 800, 96
+
+
+def split_by_chunks(ns, chunks):
+    """(orders factored in blocks, the others): units go into chunks sorted by order, largest first, here of equal
+    numbers.  With the kernel timers on a chunk is one part."""
+    blocked, rest = [], []
+    for part in np.array_split(np.sort(np.asarray(ns, dtype=int))[::-1], max(1, chunks)):
+        if len(part):
+            (blocked if part[0] >= BLOCK_N else rest).extend(int(x) for x in part)
+    return blocked, rest
 
 
 def block_update_work(ns, nb=32):
@@ -427,10 +436,10 @@ def block_update_work(ns, nb=32):
 
 
 def kernel_models(K, n_fwd, sweeps, n_delta, n_energy, fp32_ops, fp64_peak, tc_peak, hbm_gbs, precision, nb=32,
-                  sparse=None, bf16_peak=None):
+                  sparse=None, bf16_peak=None, chunks=1):
     """Algorithmic real flops per step and the matching peak (TFLOP/s) for each library kernel;
     1 complex multiply-add = 8 real flops.  n_fwd: n of every forward unit; sweeps: per-unit
-    refinement sweeps and probes of the forward and of the adjoint."""
+    refinement sweeps and probes of the forward and of the adjoint; chunks: of the factorization."""
     n = np.asarray(n_fwd, dtype=np.float64)
     S = n / K
     mixed = precision == "mixed"
@@ -441,8 +450,8 @@ def kernel_models(K, n_fwd, sweeps, n_delta, n_energy, fp32_ops, fp64_peak, tc_p
     six = bf16_peak / 6.0 if bf16_peak else tc_peak       # six bf16 products per FP32-accurate one
     fs, fp, bs, bp = sweeps
     if mixed:
-        small = [x for x in ni if x < BLOCK_N]
-        fl, by, inner, inner_by = block_update_work([x for x in ni if x >= BLOCK_N], nb)
+        blocked, small = split_by_chunks(ni, chunks)
+        fl, by, inner, inner_by = block_update_work(blocked, nb)
         if fl:
             m["k_gemm_tc96"] = (fl, six, "complex trailing update, 96 columns of L (six bf16 products); tensor peak = "
                                 "measured bf16 / 6", by)
@@ -461,6 +470,11 @@ def kernel_models(K, n_fwd, sweeps, n_delta, n_energy, fp32_ops, fp64_peak, tc_p
         m["k_solve_c64"] = (float(np.sum(8.0 * n * n * PROBES * (fp + bp))), simt_peak,
                             "triangular solves of the convergence probes (2 columns, FP32 pipe)",
                             float(np.sum(8.0 * n * n * (fp + bp))))
+        # per slice of 16 columns one read of M as double-float pairs (16 n^2)
+        sl = -(-K // 16), -(-2 * K // 16)
+        m["k_residual_tc"] = (float(np.sum(8.0 * n * n * (K * fs + 2 * K * bs))), bf16_peak / 21.0 if bf16_peak else df_peak,
+                              "FP64-accurate residual, exact bf16 digit products; tensor peak = measured bf16 / 21",
+                              float(np.sum(16.0 * n * n * (sl[0] * fs + sl[1] * bs))))
         m["k_residual"] = (float(np.sum(8.0 * n * n * (K * fs + 2 * K * bs))), df_peak,
                            "FP64-accurate residual in double-float FP32 arithmetic (44 FP32 ops per complex MAC)")
         m["k_probe_residual"] = (float(np.sum(8.0 * n * n * PROBES * (fp + bp))), df_peak,
@@ -707,7 +721,8 @@ def run_ours(args):
     sparse = sparse_product_cmacs(np.asarray(J), np.asarray(w.species), ex["offsets"], ex["site_atom"], grad_sigma,
                                   w.K)
     models = kernel_models(w.K, n_fwd, (fs, fp, bs, bp), w.n_delta, len(w.z), fp32_ops, fp64_peak, tc_peak,
-                           fpk["hbm_gbs"], args.precision, sparse=sparse, bf16_peak=fpk.get("bf16_tflops"))
+                           fpk["hbm_gbs"], args.precision, sparse=sparse, bf16_peak=fpk.get("bf16_tflops"),
+                           chunks=int(kt["k_lapack_rows"][1]) if kt and "k_lapack_rows" in kt else 1)
     rows = kernel_rows(kt, models, fpk["hbm_gbs"])
     roof = None
     modelled = [r for r in rows.values() if "frac" in r]
@@ -720,7 +735,7 @@ def run_ours(args):
         elif top["bound"] == "hbm":
             top["peak_source"] = fpk["source"]
         else:
-            top["peak_source"] = "3xTF32 = measured cuBLAS TF32 / 3 (this run)"
+            top["peak_source"] = "measured cuBLAS TF32 (this run) or bf16 rate, over the products of the kernel's form (work)"
         roof = {k: top[k] for k in ("kernel", "bound", "achieved", "peak", "unit", "frac", "traffic", "ms_per_step",
                                     "launches_per_step", "peak_source", "work") if k in top}
 

@@ -1,6 +1,6 @@
-"""The bench's work models of the trailing updates: units are counted by their own order (a few large ones do
-not turn all into blocked ones), the constants are the library's, and the updates of a block add up to those
-of an unblocked factorization's columns."""
+"""The bench's work models of the trailing updates: units are counted by their chunk's largest order (one large
+matrix turns its own chunk into a blocked one, not all), the constants are the library's, and the updates of
+a block add up to those of an unblocked factorization's columns."""
 import os
 import re
 import sys
@@ -13,9 +13,9 @@ sys.path.insert(0, ROOT)
 import bench  # noqa: E402
 
 
-def _models(ns, precision="mixed"):
-    return bench.kernel_models(16, ns, (0 * bench.np.array(ns, float),) * 4, 1, 2, 1e13, 1.1, 340.0, 6800.0, precision,
-                               bf16_peak=1900.0)
+def _models(ns, chunks=1):
+    return bench.kernel_models(16, ns, (0 * bench.np.array(ns, float),) * 4, 1, 2, 1e13, 1.1, 340.0, 6800.0, "mixed",
+                               bf16_peak=1900.0, chunks=chunks)
 
 
 def test_constants_are_the_librarys():
@@ -27,13 +27,15 @@ def test_constants_are_the_librarys():
     assert int(re.search(r"kBlkK = (\d+)", src).group(1)) == bench.BLOCK_COLS
 
 
-def test_units_are_counted_by_their_own_order():
-    small, large = [688] * 50, [944]
-    both = _models(small + large)
-    assert both["k_gemm_tc96"][0] == _models(large)["k_gemm_tc96"][0]
-    assert both["k_gemm_tc"][0] == pytest.approx(_models(small)["k_gemm_tc"][0] + _models(large)["k_gemm_tc"][0])
-    assert both["k_gemm_tc"][3] == pytest.approx(_models(small)["k_gemm_tc"][3] + _models(large)["k_gemm_tc"][3])
-    assert "k_gemm_tc96" not in _models(small)
+def test_units_are_counted_by_their_chunk():
+    ns = [688] * 50 + [944] + [720] * 49
+    assert bench.split_by_chunks(ns, 1) == ([944] + [720] * 49 + [688] * 50, [])
+    assert bench.split_by_chunks(ns, 2) == ([944] + [720] * 49, [688] * 50)
+    assert bench.split_by_chunks([688] * 3, 5) == ([], [688] * 3)
+    both, a, b = _models(ns, 2), _models([944] + [720] * 49), _models([688] * 50)
+    assert "k_gemm_tc96" not in b and both["k_gemm_tc96"][0] == pytest.approx(a["k_gemm_tc96"][0])
+    for i in (0, 3):
+        assert both["k_gemm_tc"][i] == pytest.approx(a["k_gemm_tc"][i] + b["k_gemm_tc"][i])
 
 
 @pytest.mark.parametrize("n", [800, 928, 944, 2192])
