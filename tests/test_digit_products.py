@@ -83,12 +83,11 @@ def _solve(M, B, update):
     return X
 
 
-@pytest.mark.parametrize("kind,size", [("f", 5e-3), ("f", 1e-4), ("f", 1e-8), ("atom", 6), ("atom", 12),
-                                       ("channel", 6), ("channel", 12), ("dense", 3)])
-@pytest.mark.parametrize("lmax,n_atoms", [(3, 20), (2, 33)])
-def test_digit_products_are_as_accurate_as_fp64(kind, size, lmax, n_atoms):
-    if kind == "f" and lmax < 3:
-        pytest.skip("no f states")
+@pytest.mark.parametrize("lmax,n_atoms,kind,size", [
+    (3, 20, "f", 5e-3), (3, 20, "f", 1e-4), (3, 20, "f", 1e-8)] + [
+    (lmax, n_atoms, kind, size) for lmax, n_atoms in ((3, 20), (2, 33))
+    for kind, size in (("atom", 6), ("atom", 12), ("channel", 6), ("channel", 12), ("dense", 3))])
+def test_digit_products_are_as_accurate_as_fp64(lmax, n_atoms, kind, size):
     M = graded_matrix(wl.cluster(n_atoms, lmax, seed=40 + n_atoms, spread=2.4 * n_atoms ** (1 / 3) + 4.0), kind, size)
     K = (lmax + 1) ** 2
     ref = refined(M, K)
