@@ -256,8 +256,10 @@ __global__ void __launch_bounds__(oz::NT, 1) k_gemm64_tc(const Unit* __restrict_
     const int row = row0 + ar;
     double2 v[8];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
+    for (int q = 0; q < 8; ++q)
       v[q] = row < n ? A[(size_t)(k + chunk * 8 + q) * n + row] : make_double2(0.0, 0.0);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
       const int e = __reduce_max_sync(0xffffffffu, balance_exp(exp_field(v[q])));
       if (lane == q) sKexp[(warp & 3) * NB + chunk * 8 + q] = e;
     }
