@@ -40,18 +40,18 @@ def check_unit_status(status):
 # it grows by 2 GiB at most (n = 4144, 108 units: 2.4 to 3.0 GB, 381 to 290 ms), and a Problem that is
 # not alone on the device, or close to the end of its memory, keeps the small one: the growth takes at
 # most 1 / ADJOINT_FREE_SHARE of what is free (asked for above ADJOINT_ASK_BYTES: the question takes 0.2 ms
-# of a first pass of 2.7).
+# of a first pass, 2.7 to 4 ms for problems below that).
 ADJOINT_GROWTH_BYTES = 2 << 30
 DETACHED_GROWTH_BYTES = 8 << 30  # with the factors in it and given back at once: the library's own chunk budget
 ADJOINT_FREE_SHARE = 16
-ADJOINT_ASK_BYTES = 64 << 20
+ADJOINT_ASK_BYTES = 256 << 20
 
 
-def _free_bytes(device):
-    """Device memory that PyTorch can still hand out: free on the device, or cached and unused."""
+def _is_free(need, device):
+    """Whether PyTorch can still hand out `need` bytes: free on the device, or cached and unused."""
     import torch
-    cached = torch.cuda.memory_reserved(device) - torch.cuda.memory_allocated(device)
-    return torch.cuda.mem_get_info(device)[0] + cached
+    free = torch.cuda.mem_get_info(device)[0]
+    return need <= free or need <= free + torch.cuda.memory_reserved(device) - torch.cuda.memory_allocated(device)
 
 
 class Problem:
@@ -180,7 +180,8 @@ class Problem:
         import torch
         small = min(al, max(mn, self.workspace.numel()))
         size = small if self._capped else min(al, small + growth)
-        if size - small > ADJOINT_ASK_BYTES and (size - small) * ADJOINT_FREE_SHARE > _free_bytes(self.device):
+        grow = size - small
+        if grow > ADJOINT_ASK_BYTES and not _is_free(grow * ADJOINT_FREE_SHARE, self.device):
             size = small
         try:
             return torch.empty(size, dtype=torch.uint8, device=self.device)

@@ -1,5 +1,5 @@
 """The size of the adjoint's workspace (kept by a Problem for its lifetime): all units where that is little,
-at most 2 GiB more than the forward's, and the forward's size where the growth is above 64 MiB and more than
+at most 2 GiB more than the forward's, and the forward's size where the growth is above 256 MiB and more than
 a sixteenth of the free memory, or the caller gave a cap.  Host only: the device's free memory is made up."""
 import types
 
@@ -33,5 +33,5 @@ def test_adjoint_workspace_leaves_the_rest_of_a_full_device(monkeypatch):
     assert _size(monkeypatch, 160 * MB, 161 * MB, 494 * MB, 4 * GB) == 161 * MB
     assert _size(monkeypatch, 160 * MB, 161 * MB, 494 * MB, 1 * GB, cached=20 * GB) == 494 * MB
     assert _size(monkeypatch, 3 * MB, 7 * MB, 19 * MB, 4 * GB) == 19 * MB
-    assert _size(monkeypatch, 3 * MB, 7 * MB, 71 * MB, 0) == 71 * MB  # 64 MB are taken without asking
-    assert _size(monkeypatch, 3 * MB, 7 * MB, 72 * MB, 0) == 7 * MB
+    assert _size(monkeypatch, 3 * MB, 7 * MB, 263 * MB, 0) == 263 * MB  # 256 MB are taken without asking
+    assert _size(monkeypatch, 3 * MB, 7 * MB, 264 * MB, 0) == 7 * MB
